@@ -753,42 +753,156 @@ extern "C" dgw_status dgw_rk_step_host(dgw_ctx* c, const void* U_in, void* U_out
 // ------------------------------------------------------------------------------------
 // projection
 // ------------------------------------------------------------------------------------
+// L2 projection, one thread per cell: c_ij = minv_i minv_j sum_ab w_a w_b P_i(g_a) P_j(g_b) f_ab
+// by sum factorisation, two sample rows (+-g_b) at a time.  Everything is summed in double,
+// and the FP64 pipe (2 lanes per SM) bounds the kernel, not memory: on the symmetric Gauss
+// nodes P_i(-g) = +-P_i(g), so sums over +-pairs halve the multiplications, and each sample is
+// read once: 288 FP64 operations a cell at 8 x 8 samples and p = 3.  The direct double loop over
+// modes took 2688 and read every sample K times: 1024^2 cells, 4.53 ms with the mass that follows,
+// now 0.73 ms (the 604 MB it moves would take 0.09 ms).
 struct ProjArgs {
     const double* f;
     void* U;
     int64_t E;
-    int nq, n1, dim, f64;
-    double w[8];
-    double B[8][kMaxN1];
+    int f64;
+    int vec;                        // sample rows start on 16-byte boundaries
+    double WB[8][kMaxN1];           // w_q P_i(g_q)
     double minv[kMaxN1];
 };
 
-__global__ void project_kernel(const ProjArgs a)
+// out[i] = sum_q WB[q][i] f[q] on symmetric nodes
+template <int NQ, int N1>
+__device__ __forceinline__ void proj_sum(const double (&WB)[8][kMaxN1], const double (&f)[NQ], double (&out)[N1])
 {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.E) return;
-    const int npt = a.dim == 1 ? a.nq : a.nq * a.nq;
-    const double* f = a.f + e * npt;
-    const int K = a.dim == 1 ? a.n1 : a.n1 * a.n1;
-    for (int k = 0; k < K; ++k) {
-        const int i = k % a.n1, j = k / a.n1;
-        double s = 0.0;
-        if (a.dim == 1) {
-            for (int q = 0; q < a.nq; ++q) s += a.w[q] * a.B[q][i] * f[q];
-            s *= a.minv[i];
-        } else {
-            for (int qb = 0; qb < a.nq; ++qb) {
-                double r = 0.0;
-                for (int qa = 0; qa < a.nq; ++qa) r += a.w[qa] * a.B[qa][i] * f[qa + a.nq * qb];
-                s += a.w[qb] * a.B[qb][j] * r;
-            }
-            s *= a.minv[i] * a.minv[j];
-        }
-        if (a.f64) static_cast<double*>(a.U)[k * a.E + e] = s;
-        else static_cast<float*>(a.U)[k * a.E + e] = (float)s;
+    constexpr int NP = NQ / 2;
+    double S[NP > 0 ? NP : 1], D[NP > 0 ? NP : 1];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) {
+        S[m] = f[NQ - 1 - m] + f[m];
+        D[m] = f[NQ - 1 - m] - f[m];
+    }
+#pragma unroll
+    for (int i = 0; i < N1; ++i) {
+        double a = 0.0;
+        if ((NQ & 1) != 0 && (i & 1) == 0) a = WB[NQ / 2][i] * f[NQ / 2];
+#pragma unroll
+        for (int m = 0; m < NP; ++m) a = fma(WB[NQ - 1 - m][i], (i & 1) ? D[m] : S[m], a);
+        out[i] = a;
     }
 }
 
+template <int DIM, int N1, int NQ>
+__global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ ProjArgs a)
+{
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= a.E) return;
+    constexpr int NPT = DIM == 1 ? NQ : NQ * NQ, NP = NQ / 2, K = DIM == 1 ? N1 : N1 * N1;
+    const double* f = a.f + e * NPT;
+    auto load = [&](int b, double (&r)[NQ]) {
+        const double* src = f + b * NQ;
+        if ((NQ & 1) == 0 && a.vec) {
+#pragma unroll
+            for (int q = 0; q + 1 < NQ; q += 2) {
+                const double2 v = *reinterpret_cast<const double2*>(src + q);
+                r[q] = v.x;
+                r[q + 1] = v.y;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) r[q] = src[q];
+        }
+    };
+    double c[K];
+    if constexpr (DIM == 1) {
+        double r[NQ];
+        load(0, r);
+        proj_sum<NQ, N1>(a.WB, r, c);
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k) c[k] = 0.0;
+        if constexpr ((NQ & 1) != 0) {
+            double r[NQ], s[N1];
+            load(NQ / 2, r);
+            proj_sum<NQ, N1>(a.WB, r, s);
+#pragma unroll
+            for (int j = 0; j < N1; j += 2)
+#pragma unroll
+                for (int i = 0; i < N1; ++i) c[i + N1 * j] = a.WB[NQ / 2][j] * s[i];
+        }
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {
+            double rm[NQ], rp[NQ], sm[N1], sp[N1];
+            load(m, rm);
+            load(NQ - 1 - m, rp);
+            proj_sum<NQ, N1>(a.WB, rm, sm);
+            proj_sum<NQ, N1>(a.WB, rp, sp);
+#pragma unroll
+            for (int i = 0; i < N1; ++i) {
+                const double S = sp[i] + sm[i], D = sp[i] - sm[i];
+#pragma unroll
+                for (int j = 0; j < N1; ++j)
+                    c[i + N1 * j] = fma(a.WB[NQ - 1 - m][j], (j & 1) ? D : S, c[i + N1 * j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const double v = c[k] * (DIM == 1 ? a.minv[k] : a.minv[k % N1] * a.minv[k / N1]);
+        if (a.f64) static_cast<double*>(a.U)[k * a.E + e] = v;
+        else static_cast<float*>(a.U)[k * a.E + e] = (float)v;
+    }
+}
+
+// Fills the tables for degree p and the nq-point Gauss rule (P_0..P_p by their recurrence).
+static void project_tables(ProjArgs& a, int p, int nq)
+{
+    double x[8], w[8];
+    gauss_rule_public(nq, x, w);
+    for (int q = 0; q < nq; ++q) {
+        double pm = 1.0, pc = x[q];
+        a.WB[q][0] = w[q];
+        a.WB[q][1] = w[q] * pc;
+        for (int k = 1; k < p; ++k) {
+            const double pn = ((2 * k + 1) * x[q] * pc - k * pm) / (k + 1);
+            pm = pc; pc = pn;
+            a.WB[q][k + 1] = w[q] * pn;
+        }
+    }
+    for (int i = 0; i <= p; ++i) a.minv[i] = (2 * i + 1) / 2.0;
+}
+
+template <int DIM, int N1>
+static void launch_project_n(const ProjArgs& a, int nq, unsigned blocks, cudaStream_t s)
+{
+    switch (nq) {
+    case 1: project_kernel<DIM, N1, 1><<<blocks, 128, 0, s>>>(a); break;
+    case 2: project_kernel<DIM, N1, 2><<<blocks, 128, 0, s>>>(a); break;
+    case 3: project_kernel<DIM, N1, 3><<<blocks, 128, 0, s>>>(a); break;
+    case 4: project_kernel<DIM, N1, 4><<<blocks, 128, 0, s>>>(a); break;
+    case 5: project_kernel<DIM, N1, 5><<<blocks, 128, 0, s>>>(a); break;
+    case 6: project_kernel<DIM, N1, 6><<<blocks, 128, 0, s>>>(a); break;
+    case 7: project_kernel<DIM, N1, 7><<<blocks, 128, 0, s>>>(a); break;
+    default: project_kernel<DIM, N1, 8><<<blocks, 128, 0, s>>>(a); break;
+    }
+}
+
+// Samples f (E nq^dim, nq in 1..8) to the modes of degree p in U; a's tables are filled.
+static cudaError_t launch_project(ProjArgs& a, const double* f, void* U, int64_t E, int dim, int p, int nq, cudaStream_t s)
+{
+    a.f = f; a.U = U; a.E = E;
+    a.vec = ((uintptr_t)f & 15u) == 0;       // with nq even every row starts where f does, mod 16 bytes
+    const unsigned blocks = (unsigned)((E + 127) / 128);
+    if (dim == 1) {
+        if (p == 1) launch_project_n<1, 2>(a, nq, blocks, s);
+        else if (p == 2) launch_project_n<1, 3>(a, nq, blocks, s);
+        else launch_project_n<1, 4>(a, nq, blocks, s);
+    } else {
+        if (p == 1) launch_project_n<2, 2>(a, nq, blocks, s);
+        else if (p == 2) launch_project_n<2, 3>(a, nq, blocks, s);
+        else launch_project_n<2, 4>(a, nq, blocks, s);
+    }
+    return cudaGetLastError();
+}
 
 extern "C" dgw_status dgw_project(dgw_ctx* c, int nq, const double* samples, void* U, void* stream)
 {
@@ -798,33 +912,15 @@ extern "C" dgw_status dgw_project(dgw_ctx* c, int nq, const double* samples, voi
     if (nq < 1 || nq > 8) return fail(DGW_EINVAL, "nq must lie in 1..8");
     ProjArgs a;
     std::memset(&a, 0, sizeof a);
-    a.f = samples; a.U = U; a.E = c->E; a.nq = nq; a.n1 = c->p + 1; a.dim = c->mesh.dim;
+    project_tables(a, c->p, nq);
     a.f64 = c->params.prec == DGW_FP64;
-    double x[8];
-    gauss_rule_public(nq, x, a.w);
-    for (int q = 0; q < nq; ++q) {
-        // P_0..P_p at x_q by the three-term recurrence
-        double pm = 1.0, pc = x[q];
-        a.B[q][0] = 1.0;
-        if (c->p >= 1) a.B[q][1] = x[q];
-        for (int k = 1; k < c->p; ++k) {
-            double pn = ((2 * k + 1) * x[q] * pc - k * pm) / (k + 1);
-            pm = pc; pc = pn;
-            a.B[q][k + 1] = pn;
-        }
-    }
-    for (int i = 0; i <= c->p; ++i) a.minv[i] = (2 * i + 1) / 2.0;
-    const int threads = 128;
-    const int64_t blocks = (c->E + threads - 1) / threads;
     // the Euler system: one projection per component (samples and rows component-major)
     const int ncomp = c->flux.kind == DGW_FLUX_EULER ? c->mesh.dim + 2 : 1;
     const int64_t npt = c->mesh.dim == 1 ? nq : nq * nq;
-    for (int comp = 0; comp < ncomp; ++comp) {
-        a.f = samples + comp * c->E * npt;
-        a.U = static_cast<char*>(U) + (size_t)comp * (c->K / ncomp) * c->E * c->eb;
-        project_kernel<<<(unsigned)blocks, threads, 0, (cudaStream_t)stream>>>(a);
-        DGW_CUDA(cudaGetLastError());
-    }
+    for (int comp = 0; comp < ncomp; ++comp)
+        DGW_CUDA(launch_project(a, samples + comp * c->E * npt,
+                                static_cast<char*>(U) + (size_t)comp * (c->K / ncomp) * c->E * c->eb, c->E, c->mesh.dim,
+                                c->p, nq, (cudaStream_t)stream));
     return DGW_OK;
 }
 
@@ -1077,31 +1173,16 @@ extern "C" dgw_status dgw_batch_project(dgw_batch* b, int nq, int first, int cou
     if (!b || !samples || !U) return fail(DGW_EINVAL, "NULL argument");
     if (nq < 1 || nq > 8) return fail(DGW_EINVAL, "nq must lie in 1..8");
     if (first < 0 || count < 0 || first + count > b->n) return fail(DGW_EINVAL, "instance range out of bounds");
-    double x[8], w[8];
-    gauss_rule_public(nq, x, w);
+    ProjArgs a;
+    std::memset(&a, 0, sizeof a);
+    a.f64 = b->eb == 8;
     int64_t so = 0;
     for (int i = first; i < first + count; ++i) {
         const BatchInst& I = b->inst[i];
-        ProjArgs a;
-        std::memset(&a, 0, sizeof a);
-        a.f = samples + so;
+        project_tables(a, I.p, nq);
+        DGW_CUDA(launch_project(a, samples + so, static_cast<char*>(U) + (size_t)I.off * b->eb, I.E, b->dims[i], I.p,
+                                nq, (cudaStream_t)stream));
         so += I.E * (b->dims[i] == 1 ? nq : nq * nq);
-        a.U = static_cast<char*>(U) + (size_t)I.off * b->eb;
-        a.E = I.E; a.nq = nq; a.n1 = I.p + 1; a.dim = b->dims[i]; a.f64 = b->eb == 8;
-        for (int q = 0; q < nq; ++q) {
-            a.w[q] = w[q];
-            double pm = 1.0, pc = x[q];
-            a.B[q][0] = 1.0;
-            a.B[q][1] = x[q];
-            for (int k = 1; k < I.p; ++k) {
-                double pn = ((2 * k + 1) * x[q] * pc - k * pm) / (k + 1);
-                pm = pc; pc = pn;
-                a.B[q][k + 1] = pn;
-            }
-        }
-        for (int k = 0; k <= I.p; ++k) a.minv[k] = (2 * k + 1) / 2.0;
-        project_kernel<<<(unsigned)((I.E + 127) / 128), 128, 0, (cudaStream_t)stream>>>(a);
-        DGW_CUDA(cudaGetLastError());
     }
     return DGW_OK;
 }
