@@ -178,37 +178,55 @@ __device__ __forceinline__ double mul_x(double a, double b) { return __dmul_rn(a
 __device__ __forceinline__ float fma_x(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_x(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// Flux F(u) at (x, y) and |F'(u)|_2 (1D: only the x component).
+// Flux F(u) at (x, y) (1D: only the x component) and the key by which |F'(u)|_2 is compared
+// over a cell's points: a quantity that grows with |F'(u)|_2, so that the largest key gives
+// lambda_e through one speed_of_key per cell.  Advection: none (0; the speed is constant);
+// rotation: |F'|^2 in 2D; Burgers: |u|; KPP: |F'| itself.  The square root and the product are
+// monotone in floating point too, so lambda_e has the same bits as the maximum of the points'
+// speeds.  It pays most in double, where a root costs about 25 operations of a pipe that has 2
+// lanes per SM: rotation at 256^2 Q2, FP64, 181 -> 151 us a stage; the float ensemble of 2D
+// advection (no keys at its faces any more) 2.50 -> 2.29 ms a step.
 template <int FLUX>
 __device__ __forceinline__ void vol_flux(const KParams& A, Real u, Real x, Real y, Real& fx, Real& fy,
-                                         Real& spd)
+                                         Real& key)
 {
     if (FLUX == FLUX_ADVECT) {
         fx = mul_x(A.a0, u); fy = mul_x(A.a1, u);
-        spd = DIM == 1 ? fabs(A.a0) : sqrt_r(fma_x(A.a0, A.a0, mul_x(A.a1, A.a1)));
+        key = Real(0);
     } else if (FLUX == FLUX_ROTATION) {
         const Real vx = mul_x(A.omega, A.cy - y), vy = mul_x(A.omega, x - A.cx);
         fx = mul_x(vx, u); fy = mul_x(vy, u);
-        spd = DIM == 1 ? fabs(vx) : sqrt_r(fma_x(vx, vx, mul_x(vy, vy)));
+        key = DIM == 1 ? fabs(vx) : fma_x(vx, vx, mul_x(vy, vy));
     } else if (FLUX == FLUX_BURGERS) {
         const Real hu2 = mul_x(mul_x(Real(0.5), u), u);
         fx = mul_x(A.a0, hu2); fy = mul_x(A.a1, hu2);
-        spd = DIM == 1 ? fabs(mul_x(A.a0, u)) : mul_x(sqrt_r(fma_x(A.a0, A.a0, mul_x(A.a1, A.a1))), fabs(u));
+        key = fabs(u);
     } else {  // KPP: F = (sin u, cos u), |F'| = 1 in 2D
         Real s, c;
         sincos_r(u, &s, &c);
         fx = s; fy = c;
-        spd = DIM == 1 ? fabs(c) : Real(1);
+        key = DIM == 1 ? fabs(c) : Real(1);
     }
 }
 
 template <int FLUX>
-__device__ __forceinline__ Real speed_norm(const KParams& A, Real u, Real x, Real y)
+__device__ __forceinline__ Real speed_key(const KParams& A, Real u, Real x, Real y)
 {
     if (FLUX == FLUX_KPP && DIM == 2) return Real(1);
-    Real fx, fy, spd;
-    vol_flux<FLUX>(A, u, x, y, fx, fy, spd);
-    return spd;
+    Real fx, fy, key;
+    vol_flux<FLUX>(A, u, x, y, fx, fy, key);
+    return key;
+}
+
+template <int FLUX>
+__device__ __forceinline__ Real speed_of_key(const KParams& A, Real key)
+{
+    if (FLUX == FLUX_ADVECT || FLUX == FLUX_BURGERS) {
+        const Real a = DIM == 1 ? fabs(A.a0) : sqrt_r(fma_x(A.a0, A.a0, mul_x(A.a1, A.a1)));
+        return FLUX == FLUX_ADVECT ? a : mul_x(a, key);
+    }
+    if (FLUX == FLUX_ROTATION && DIM == 2) return sqrt_r(key);
+    return key;
 }
 
 // ------------------------------------------------------------------------------------
@@ -262,15 +280,15 @@ __device__ __forceinline__ void sincos_v(Real x, Real& s, Real& c) { sincos_r(x,
 __device__ __forceinline__ void sincos_v(float2 x, float2& s, float2& c) { fast_sincos2(x, &s, &c); }
 
 template <int FLUX, class V>
-__device__ __forceinline__ void vol_flux_v(const KParams& A, V u, Real x, V y, V& fx, V& fy, V& spd)
+__device__ __forceinline__ void vol_flux_v(const KParams& A, V u, Real x, V y, V& fx, V& fy, V& key)
 {
     if constexpr (FLUX == FLUX_KPP) {
         sincos_v(u, fx, fy);
 #pragma unroll
-        for (int l = 0; l < Lanes<V>::n; ++l) lane(spd, l) = DIM == 1 ? fabs(lane(fy, l)) : Real(1);
+        for (int l = 0; l < Lanes<V>::n; ++l) lane(key, l) = DIM == 1 ? fabs(lane(fy, l)) : Real(1);
     } else {
 #pragma unroll
-        for (int l = 0; l < Lanes<V>::n; ++l) vol_flux<FLUX>(A, lane(u, l), x, lane(y, l), lane(fx, l), lane(fy, l), lane(spd, l));
+        for (int l = 0; l < Lanes<V>::n; ++l) vol_flux<FLUX>(A, lane(u, l), x, lane(y, l), lane(fx, l), lane(fy, l), lane(key, l));
     }
 }
 
@@ -606,7 +624,11 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
 
     const int tid = threadIdx.x;
     const int64_t E = A.E;
-    const bool need_lam = (MODE == 0) && (A.stab != STAB_DG) && !A.lam_fixed;
+    // lambda_e from the largest key of the cell's points; advection and the 2D KPP flux have the
+    // same key at every point, so their faces contribute nothing
+    constexpr bool kSameSpeed = FLUX == FLUX_ADVECT || (FLUX == FLUX_KPP && DIM == 2);
+    const bool find_lam = (MODE == 0) && (A.stab != STAB_DG) && !A.lam_fixed;
+    const bool need_lam = find_lam && !kSameSpeed;
     const bool periodic_x = A.bc[0] == BC_PERIODIC;
     const bool periodic_y = DIM == 2 && A.bc[2] == BC_PERIODIC;
 
@@ -887,7 +909,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     V acc[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = vbc<V>(0);
-    V lam = vbc<V>(0);
+    V lam = vbc<V>(0);        // largest key of the cell's points (vol_flux)
     const Real xc = fma_x(Real(gx) + Real(0.5), A.h, A.x0);
     V yc;
 #pragma unroll
@@ -897,9 +919,9 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
         interp_sym<N1, NQ>(T.B, c, u);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            V fy, spd;
-            vol_flux_v<FLUX>(A, u[q], fma_x(A.hh, T.g[q], xc), vbc<V>(0), fx[q], fy, spd);
-            lam = vmax(lam, spd);
+            V fy, key;
+            vol_flux_v<FLUX>(A, u[q], fma_x(A.hh, T.g[q], xc), vbc<V>(0), fx[q], fy, key);
+            lam = vmax(lam, key);
         }
         project_sym<true, N1, NQ>(T.WD, fx, acc);
         acc[0] = vbc<V>(0);
@@ -916,9 +938,9 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             interp_sym<N1, NQ>(T.B, rr, u);
 #pragma unroll
             for (int qx = 0; qx < NQ; ++qx) {
-                V spd;
-                vol_flux_v<FLUX>(A, u[qx], fma_x(A.hh, T.g[qx], xc), y, fx[qx], fy[qx], spd);
-                lam = vmax(lam, spd);
+                V key;
+                vol_flux_v<FLUX>(A, u[qx], fma_x(A.hh, T.g[qx], xc), y, fx[qx], fy[qx], key);
+                lam = vmax(lam, key);
             }
             V px[N1], py[N1];
             project_sym<true, N1, NQ>(T.WD, fx, px);      // px[0] = 0 (P_0' = 0)
@@ -1068,8 +1090,8 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                 if (need_lam) {
 #pragma unroll
                     for (int l = 0; l < L; ++l) {   // |F'| = 1 in 2D; 1D: |cos u| (no shift)
-                        lane(lm, l) = fmax(lane(lm, l), speed_norm<FLUX>(A, lane(uL, l), Real(0), Real(0)));
-                        lane(lp, l) = fmax(lane(lp, l), speed_norm<FLUX>(A, lane(uR, l), Real(0), Real(0)));
+                        lane(lm, l) = fmax(lane(lm, l), speed_key<FLUX>(A, lane(uL, l), Real(0), Real(0)));
+                        lane(lp, l) = fmax(lane(lp, l), speed_key<FLUX>(A, lane(uR, l), Real(0), Real(0)));
                     }
                 }
                 Hq[q] = llf_kpp(uL, uR);
@@ -1097,8 +1119,8 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                         ur = (A.bc[bside] == BC_INFLOW_ZERO && dflux_axis<FLUX>(A, axis, ul, x, y) < Real(0)) ? Real(0) : ul;
                     }
                     if (need_lam) {
-                        lane(lm, l) = fmax(lane(lm, l), speed_norm<FLUX>(A, ul, x, y));
-                        lane(lp, l) = fmax(lane(lp, l), speed_norm<FLUX>(A, ur, x, y));
+                        lane(lm, l) = fmax(lane(lm, l), speed_key<FLUX>(A, ul, x, y));
+                        lane(lp, l) = fmax(lane(lp, l), speed_key<FLUX>(A, ur, x, y));
                     }
                     lane(Hq[q], l) = llf<FLUX>(A, axis, ul, ur, x, y);
                 }
@@ -1173,9 +1195,10 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             }
         }
     }
-    if (need_lam) {
+    if (find_lam) {
 #pragma unroll
-        for (int l = 0; l < L; ++l) lane(lam, l) = fmax(lane(lam, l), lam_s[cy[l]][lx]);
+        for (int l = 0; l < L; ++l)
+            lane(lam, l) = speed_of_key<FLUX>(A, need_lam ? fmax(lane(lam, l), lam_s[cy[l]][lx]) : lane(lam, l));
     }
 
     // stabilization (Sec. 3), M^{-1}, RK combination (Eq. ssp)
