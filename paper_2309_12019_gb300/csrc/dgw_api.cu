@@ -504,11 +504,23 @@ static cudaError_t enqueue_steps_rk24(const dgw_ctx* c, void* U, double dt, int 
     return cudaSuccess;
 }
 
+// 1D meshes that fit one thread-block cluster take all their steps in one launch
+// (dgw_line_impl.cuh); nsteps = 0 asks whether c's does.
+static cudaError_t line_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
+{
+    if (c->mesh.dim != 1) return cudaErrorNotSupported;
+    const StageArgs a = base_args(c);
+    return c->eb == 8 ? launch_line_f64_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s)
+                      : launch_line_f32_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s);
+}
+
 // One SSP-RK3 step (Eq. ssp): U1 = U + dt L(U); U2 = 3/4 U + 1/4 (U1 + dt L(U1));
 // U <- 1/3 U + 2/3 (U2 + dt L(U2)).  The third stage writes U in place: each thread
 // reads U only at its own element there.  Other orders: enqueue_steps_rk24.
 static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
+    const cudaError_t le = line_steps(c, U, dt, nsteps, s);
+    if (le != cudaErrorNotSupported) return le;
     if (c->params.rk_order != 3) return enqueue_steps_rk24(c, U, dt, nsteps, s);
     StageArgs a = base_args(c);
     for (int n = 0; n < nsteps; ++n) {
@@ -574,7 +586,7 @@ extern "C" dgw_status dgw_rk_step(dgw_ctx* c, void* U, double dt, int nsteps, vo
     cudaStream_t s = (cudaStream_t)stream;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (s != nullptr) DGW_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (s == nullptr || cap != cudaStreamCaptureStatusNone) {
+    if (s == nullptr || cap != cudaStreamCaptureStatusNone || line_steps(c, U, dt, 0, s) == cudaSuccess) {
         DGW_CUDA(enqueue_steps(c, U, dt, nsteps, s));
         return DGW_OK;
     }

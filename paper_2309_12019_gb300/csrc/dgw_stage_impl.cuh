@@ -1763,6 +1763,7 @@ __device__ __forceinline__ Real max_nan(Real a, Real b)
 
 #if DGW_DIM == 1
 #include "dgw_euler_impl.cuh"
+#include "dgw_line_impl.cuh"
 #else
 #include "dgw_euler2d_impl.cuh"
 #endif

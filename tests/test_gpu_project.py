@@ -20,7 +20,14 @@ def test_project_all_rules(dim, nx, ny, nq):
     for p in (1, 2, 3):
         s = H.spec(dim, p, nx, ny=ny)
         f = rng.standard_normal(nx * ny * nq ** dim)
-        want = O.project(O.Problem(**s), f, nq)
+        # the rule's sums in NumPy (the oracle divides by the rule's own norm of P_i, which is the
+        # exact one from p + 1 points on)
+        g, w = np.polynomial.legendre.leggauss(nq)
+        M = np.polynomial.legendre.legvander(g, p) * w[:, None] * (np.arange(p + 1) + 0.5)
+        v = f.reshape((nx * ny,) + (nq,) * dim)
+        want = np.einsum("ea,ai->ie", v, M) if dim == 1 else np.einsum("eba,ai,bj->jie", v, M, M).reshape(-1, nx * ny)
+        if nq > p:
+            assert np.allclose(want, O.project(O.Problem(**s), f, nq), rtol=0, atol=1e-12)
         # |sum w_a w_b P_i P_j f| <= 4 max |f|, times minv_i minv_j <= 12.25; at most 20 roundings of
         # partial sums in double on either side, and one of the result in float
         tol = {"fp64": 2 * 20 * 4 * 2.0 ** -53, "fp32": 4 * 2.0 ** -24}
