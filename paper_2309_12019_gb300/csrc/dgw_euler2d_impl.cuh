@@ -4,7 +4,7 @@
 //
 // State U = (rho, rho vx, rho vy, rho E), p = (gamma - 1)(rho E - rho |v|^2 / 2); mode
 // k = i + (p+1) j of component comp of cell e at row comp K + k, K = (p+1)^2.
-// One CTA of EX x EY = 32 x 4 threads owns a tile of as many cells, one per thread:
+// One CTA of 32 x EY threads owns a tile of as many cells, one per thread:
 //   0. the tile's coefficients and a one-cell face halo (all four components) are
 //      staged in shared memory by coalesced row loads; halo cells beyond a periodic side
 //      are its images, beyond a wall or an outflow side they are absent; in float the
@@ -20,13 +20,20 @@
 // Constants are folded as in the scalar kernel:
 //   L_k = (2/h) minv(i) minv(j) [acc_k - gamma lambda / p (K_ref c)_k].
 
-constexpr int EX = kTileX2, EY = kTileY2, ENT = EX * EY;
+// Tile heights: 8 rows (256 threads, two CTAs per SM) in float up to p = 2, else 4.  The kernel is
+// bound by instruction issue and by the latency of its dependent operations, so it wants warps:
+// with the tile's Un in shared memory 3 CTAs of 4 rows fitted (12 warps, issue active 59 %); Un
+// is now prefetched into L2 and read into registers after the faces, which makes room for 16
+// warps, and the taller tile has fewer halo cells and faces per cell.  Kelvin-Helmholtz 2048^2, p = 2,
+// FP32: 746 -> 680 us a stage; triple point 896 x 384: 69 -> 66 us.
 using R2 = std::conditional_t<kF32, float2, double2>;   // a pair of state components
-constexpr int EHX = EX + 2, EHY = EY + 2;          // staged columns / rows (one halo cell)
+constexpr int EX = kTileX2, EHX = EX + 2;               // tile columns, staged columns
+template <int P> constexpr int euler2_rows() { return kF32 && P <= 2 ? 8 : kTileY2; }
+template <int P> constexpr int euler2_blocks() { return 2; }
 
 template <int P>
 struct Euler2Smem {
-    static constexpr int N1 = P + 1, K = N1 * N1;
+    static constexpr int N1 = P + 1, K = N1 * N1, EY = euler2_rows<P>(), EHY = EY + 2;
     // the four components as two pairs (rho, rho vx), (rho vy, rho E), each pair one
     // 8-byte (float) or 16-byte (double) word, so that a pair is one shared load or store
     R2 u[2][K][EHY][EHX];           // coefficients; tile cell (lx, ly) at [ly + 1][lx + 1]
@@ -35,9 +42,6 @@ struct Euler2Smem {
     Real sx[2][EY][EX + 1];         // max |v| + c of the minus (0) / plus (1) cell's own values on x-face f
     Real sy[2][EY + 1][EX];         // the same on y-face r
     int has[EHY][EHX];              // the staged cell exists
-    // float: Un of the tile's cells, brought in by cp.async (in double this would halve
-    // the CTAs per SM; double reads Un at the end)
-    R2 un[kF32 ? 2 : 1][kF32 ? K : 1][EY][EX];
 };
 
 struct Euler2State {
@@ -151,9 +155,10 @@ __device__ __forceinline__ Real sensor_2d(const KParams& A, const Tab<P>& T, con
 
 // MODE 0: stage / residual; MODE 1: sensor only (writes gamma_out).
 template <int P, int MODE>
-__global__ void __launch_bounds__(ENT, (P == 3 || !kF32) ? 2 : 3) euler2d_kernel(const __grid_constant__ KParams A)
+__global__ void __launch_bounds__(EX * euler2_rows<P>(), euler2_blocks<P>()) euler2d_kernel(const __grid_constant__ KParams A)
 {
     constexpr int N1 = P + 1, NQ = P + 2, K = N1 * N1;
+    constexpr int EY = euler2_rows<P>(), ENT = EX * EY, EHY = EY + 2;
     extern __shared__ __align__(16) unsigned char smem_e2[];
     Euler2Smem<P>& S = *reinterpret_cast<Euler2Smem<P>*>(smem_e2);
     const Tab<P>& T = tab<P>();
@@ -169,29 +174,31 @@ __global__ void __launch_bounds__(ENT, (P == 3 || !kF32) ? 2 : 3) euler2d_kernel
         S.has[r][cc] = ok;
         const Real* src = A.Uk + (ok ? (int64_t)gy * A.nx + gx : 0);
 #pragma unroll
-        for (int comp = 0; comp < 4; ++comp)
+        for (int pr = 0; pr < 2; ++pr)
 #pragma unroll
-            for (int k = 0; k < K; ++k) lane(S.u[comp >> 1][k][r][cc], comp & 1) = ok ? src[(int64_t)(comp * K + k) * E] : Real(0);
+            for (int k = 0; k < K; ++k) {
+                R2 v = vbc<R2>(0);
+                if (ok) {
+                    v.x = src[(int64_t)(2 * pr * K + k) * E];
+                    v.y = src[(int64_t)((2 * pr + 1) * K + k) * E];
+                }
+                S.u[pr][k][r][cc] = v;
+            }
     }
     const int lx = tid % EX, ly = tid / EX;
     const int gx = tx0 + lx, gy = ty0 + ly;
     const bool in = gx < A.nx && gy < A.ny;
     const int64_t e = (int64_t)gy * A.nx + gx;
-    // Un is read only by the final combination: each thread starts asynchronous copies
-    // of its cell's Un coefficients into shared memory now (cp.async holds no
-    // registers) and waits for them just before that combination
-    const bool copy_un = kF32 && MODE == 0 && A.has_un && in;
-    if (copy_un) {
-#pragma unroll
-        for (int comp = 0; comp < 4; ++comp)
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&lane(S.un[kF32 ? comp >> 1 : 0][kF32 ? k : 0][ly][lx], comp & 1));
-                const Real* src = A.Un + e + (int64_t)(comp * K + k) * E;
-                asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" :: "r"(dst), "l"(src), "n"((int)sizeof(Real))
-                             : "memory");
-            }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    // Un is read after the faces: each warp asks now for its row of every coefficient (a lane
+    // per coefficient; a row that starts inside a 128-byte line ends in the next one)
+    const bool use_un = MODE == 0 && A.has_un;
+    if (use_un && gy < A.ny) {
+        const int last = (A.nx - tx0 < EX ? A.nx - tx0 : EX) - 1;
+        for (int row = lx; row < 4 * K; row += EX) {
+            const Real* a = A.Un + (int64_t)row * E + (int64_t)gy * A.nx + tx0;
+            asm volatile("prefetch.global.L2 [%0];" :: "l"(a));
+            if (((uintptr_t)a & 127u) != 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(a + last));
+        }
     }
     __syncthreads();
 
@@ -387,6 +394,19 @@ __global__ void __launch_bounds__(ENT, (P == 3 || !kF32) ? 2 : 3) euler2d_kernel
             S.sy[1][fr][fc] = spp;
         }
     }
+    // Un (float: all of it before the barrier, whose wait hides the loads; in double the
+    // registers would not hold it)
+    R2 un[kF32 ? 2 : 1][kF32 ? K : 1];
+    if (kF32 && use_un && in) {
+#pragma unroll
+        for (int pr = 0; pr < (kF32 ? 2 : 1); ++pr)
+#pragma unroll
+            for (int k = 0; k < (kF32 ? K : 1); ++k) {
+                const Real* a0 = A.Un + e + (int64_t)(2 * pr * K + k) * E;
+                un[pr][k].x = a0[0];
+                un[pr][k].y = a0[(int64_t)K * E];
+            }
+    }
     __syncthreads();
     if (!in) return;
 
@@ -396,7 +416,6 @@ __global__ void __launch_bounds__(ENT, (P == 3 || !kF32) ? 2 : 3) euler2d_kernel
                                    max_nan(S.sy[1][ly][lx], S.sy[0][ly + 1][lx])));
     const Real ngs = A.stab == STAB_DG ? Real(0) : -(gamma * (A.lam_fixed ? A.lambda_nu : lam) * Real(1.0 / P));
     Real chk = Real(0);
-    if (copy_un) asm volatile("cp.async.wait_all;" ::: "memory");   // this thread's own copies
 #pragma unroll
     for (int pr = 0; pr < 2; ++pr) {
 #pragma unroll
@@ -426,7 +445,7 @@ __global__ void __launch_bounds__(ENT, (P == 3 || !kF32) ? 2 : 3) euler2d_kernel
             if (A.has_un) {
                 R2 unk;
                 if constexpr (kF32) {
-                    unk = S.un[pr][k][ly][lx];
+                    unk = un[pr][k];
                 } else {
                     const Real* a0 = A.Un + e + (int64_t)(2 * pr * K + k) * E;
                     const Real* a1 = a0 + (int64_t)K * E;
@@ -447,6 +466,7 @@ template <int P>
 static cudaError_t launch_euler2d_p(const StageArgs& s, int mode, cudaStream_t st)
 {
     const KParams a = make_params(s);
+    constexpr int EY = euler2_rows<P>(), ENT = EX * EY;
     dim3 grid((s.nx + EX - 1) / EX, (s.ny + EY - 1) / EY);
     if (grid.x == 0 || grid.y == 0) return cudaSuccess;
     const size_t smem = sizeof(Euler2Smem<P>);
