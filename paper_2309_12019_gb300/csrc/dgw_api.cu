@@ -461,6 +461,7 @@ __global__ void rk4_mix_kernel(Real* __restrict__ q2, Real* __restrict__ q1, int
 static cudaError_t enqueue_steps_rk24(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
     StageArgs a = base_args(c);
+    a.pdl = 1;
     for (int n = 0; n < nsteps; ++n) {
         if (c->params.rk_order == 2) {
             a.Uk = U; a.Un = nullptr; a.Uout = c->S1;
@@ -523,6 +524,7 @@ static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nstep
     if (le != cudaErrorNotSupported) return le;
     if (c->params.rk_order != 3) return enqueue_steps_rk24(c, U, dt, nsteps, s);
     StageArgs a = base_args(c);
+    a.pdl = 1;
     for (int n = 0; n < nsteps; ++n) {
         a.Uk = U; a.Un = nullptr; a.Uout = c->S1;
         a.cn = 0.0; a.ck = 1.0; a.cl = dt; a.t_off = 0.0;
@@ -1462,6 +1464,7 @@ static cudaError_t vjp_combine(const dgw_ctx* c, const void* U, const void* lam,
                                cudaStream_t s)
 {
     StageArgs a = base_args(c);
+    a.pdl = 1;
     a.Uk = U;
     const bool f64 = c->params.prec == DGW_FP64;
     const int d = c->mesh.dim;
@@ -1478,6 +1481,7 @@ static cudaError_t vjp_combine(const dgw_ctx* c, const void* U, const void* lam,
     g.coef[0] = c0; g.coef[1] = c1; g.coef[2] = c2;
     g.cvjp = cv;
     g.out = out;
+    g.pdl = 1;
     return f64 ? (d == 1 ? launch_gather_f64_d1(g, c->p, s) : launch_gather_f64_d2(g, c->p, s))
                : (d == 1 ? launch_gather_f32_d1(g, c->p, s) : launch_gather_f32_d2(g, c->p, s));
 }
@@ -1512,6 +1516,7 @@ extern "C" dgw_status dgw_adjoint_step(dgw_ctx* c, const void* U_n, const void* 
     if (st != DGW_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     StageArgs a = base_args(c);
+    a.pdl = 1;
     a.Uk = U_n; a.Un = nullptr; a.Uout = c->S1;
     a.cn = 0.0; a.ck = 1.0; a.cl = dt;
     DGW_CUDA(launch(c, a, 0, s));
@@ -1541,6 +1546,7 @@ extern "C" dgw_status dgw_rk_step_stages(dgw_ctx* c, const void* U, double dt, v
     if (c->state_sides) return fail(DGW_EUNSUPPORTED, "dgw_rk_step_stages keeps no time (prescribed-state sides)");
     cudaStream_t s = (cudaStream_t)stream;
     StageArgs a = base_args(c);
+    a.pdl = 1;
     a.Uk = U; a.Un = nullptr; a.Uout = U1;
     a.cn = 0.0; a.ck = 1.0; a.cl = dt;
     DGW_CUDA(launch(c, a, 0, s));

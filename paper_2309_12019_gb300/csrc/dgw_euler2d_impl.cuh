@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(EX * euler2_rows<P>(), euler2_blocks<P>()) eul
 {
     constexpr int N1 = P + 1, NQ = P + 2, K = N1 * N1;
     constexpr int EY = euler2_rows<P>(), ENT = EX * EY, EHY = EY + 2;
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_e2[];
     Euler2Smem<P>& S = *reinterpret_cast<Euler2Smem<P>*>(smem_e2);
     const Tab<P>& T = tab<P>();
@@ -478,9 +479,7 @@ static cudaError_t launch_euler2d_p(const StageArgs& s, int mode, cudaStream_t s
         if (e != cudaSuccess) return e;
         opted[dev][mode] = true;
     }
-    if (mode == 0) euler2d_kernel<P, 0><<<grid, ENT, smem, st>>>(a);
-    else euler2d_kernel<P, 1><<<grid, ENT, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_k(mode == 0 ? euler2d_kernel<P, 0> : euler2d_kernel<P, 1>, grid, ENT, smem, s.pdl != 0, st, a);
 }
 
 static cudaError_t launch_euler2d(const StageArgs& s, int p, int mode, cudaStream_t st)

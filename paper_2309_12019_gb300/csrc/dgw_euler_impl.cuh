@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(TX, kF32 ? 8 : 4) euler_kernel(const __grid_co
 {
     constexpr int N1 = P + 1, NQ = P + 2;
     __shared__ EulerSmem<P> S;
+    pdl_begin();
     const Tab<P>& T = tab<P>();
     const int tid = threadIdx.x;
     const int64_t E = A.E;
@@ -305,9 +306,7 @@ static cudaError_t launch_euler_p(const StageArgs& s, int mode, cudaStream_t st)
     const KParams a = make_params(s);
     const unsigned grid = (unsigned)((s.nx + TX - 1) / TX);
     if (grid == 0) return cudaSuccess;
-    if (mode == 0) euler_kernel<P, 0><<<grid, TX, 0, st>>>(a);
-    else euler_kernel<P, 1><<<grid, TX, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_k(mode == 0 ? euler_kernel<P, 0> : euler_kernel<P, 1>, grid, TX, 0, s.pdl != 0, st, a);
 }
 
 static cudaError_t launch_euler(const StageArgs& s, int p, int mode, cudaStream_t st)

@@ -80,6 +80,8 @@ struct StageArgs {
     int kernel_choice;     // whole-mesh float 2D stages: 0 automatic, 1 tile kernel, 2 persistent kernel
     int tile_row0;         // 2D: first tile row of the launch
     int tile_rows;         // 2D: tile rows of the launch (0: through the last row of the mesh)
+    int pdl;               // 1: the launch may begin while the kernel before it in its stream drains
+                           // (programmatic dependent launch; sequences of whole-mesh stages)
     int wait_limit;        // polls of a bounded TMA wait: 0 the default limit, < 0 none (the
                            // wait gives up at once; diagnostic)
     // prescribed-state sides (2D Euler, DGW_BC_STATE): the stage's time is *t_dev + t_off
@@ -137,6 +139,7 @@ struct GatherArgs {
     double coef[3];
     double cvjp;
     void* out;
+    int pdl;               // as in StageArgs
 };
 
 // Launchers, one per (precision, dimension) translation unit.  mode 0: stage or
