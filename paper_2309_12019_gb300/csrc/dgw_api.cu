@@ -768,12 +768,13 @@ extern "C" dgw_status dgw_rk_step_host(dgw_ctx* c, const void* U_in, void* U_out
 // projection
 // ------------------------------------------------------------------------------------
 // L2 projection, one thread per cell: c_ij = minv_i minv_j sum_ab w_a w_b P_i(g_a) P_j(g_b) f_ab
-// by sum factorisation, two sample rows (+-g_b) at a time.  Everything is summed in double,
-// and the FP64 pipe (2 lanes per SM) bounds the kernel, not memory: on the symmetric Gauss
-// nodes P_i(-g) = +-P_i(g), so sums over +-pairs halve the multiplications, and each sample is
-// read once: 288 FP64 operations a cell at 8 x 8 samples and p = 3.  The direct double loop over
-// modes took 2688 and read every sample K times: 1024^2 cells, 4.53 ms with the mass that follows,
-// now 0.73 ms (the 604 MB it moves would take 0.09 ms).
+// by sum factorisation, two sample rows (+-g_b) at a time, each sample read once.  On the
+// symmetric Gauss nodes P_i(-g) = +-P_i(g), so sums over +-pairs halve the multiplications.
+// Double states and 1D: the sums in double, 288 operations a cell at 8 x 8 samples and p = 3; the
+// FP64 pipe (2 lanes per SM) bounds them, not memory.  Float states in 2D: project_split_kernel.
+// 1024^2 cells, p = 3, 8 x 8 samples, with the mass that follows: the direct double loop over modes
+// (2688 operations, every sample read K times) took 4.53 ms, this in double 0.73 ms, split
+// 0.20 ms (the 604 MB it moves would take 0.09 ms).
 struct ProjArgs {
     const double* f;
     void* U;
@@ -782,6 +783,7 @@ struct ProjArgs {
     int vec;                        // sample rows start on 16-byte boundaries
     double WB[8][kMaxN1];           // w_q P_i(g_q)
     double minv[kMaxN1];
+    float sh[8][kMaxN1], sl[8][kMaxN1];   // minv_i w_q P_i(g_q) = sh + sl to 48 bits
 };
 
 // out[i] = sum_q WB[q][i] f[q] on symmetric nodes
@@ -805,38 +807,41 @@ __device__ __forceinline__ void proj_sum(const double (&WB)[8][kMaxN1], const do
     }
 }
 
-template <int DIM, int N1, int NQ>
-__global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ ProjArgs a)
+// Sample row b of a cell's NPT samples f
+template <int NQ>
+__device__ __forceinline__ void proj_row(const double* f, int b, bool vec, double (&r)[NQ])
 {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= a.E) return;
+    const double* src = f + b * NQ;
+    if ((NQ & 1) == 0 && vec) {
+#pragma unroll
+        for (int q = 0; q + 1 < NQ; q += 2) {
+            const double2 v = *reinterpret_cast<const double2*>(src + q);
+            r[q] = v.x;
+            r[q + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) r[q] = src[q];
+    }
+}
+
+// The modes of cell e in double, stored in the state's precision
+template <int DIM, int N1, int NQ>
+__device__ void project_cell(const ProjArgs& a, const int64_t e)
+{
     constexpr int NPT = DIM == 1 ? NQ : NQ * NQ, NP = NQ / 2, K = DIM == 1 ? N1 : N1 * N1;
     const double* f = a.f + e * NPT;
-    auto load = [&](int b, double (&r)[NQ]) {
-        const double* src = f + b * NQ;
-        if ((NQ & 1) == 0 && a.vec) {
-#pragma unroll
-            for (int q = 0; q + 1 < NQ; q += 2) {
-                const double2 v = *reinterpret_cast<const double2*>(src + q);
-                r[q] = v.x;
-                r[q + 1] = v.y;
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) r[q] = src[q];
-        }
-    };
     double c[K];
     if constexpr (DIM == 1) {
         double r[NQ];
-        load(0, r);
+        proj_row<NQ>(f, 0, a.vec, r);
         proj_sum<NQ, N1>(a.WB, r, c);
     } else {
 #pragma unroll
         for (int k = 0; k < K; ++k) c[k] = 0.0;
         if constexpr ((NQ & 1) != 0) {
             double r[NQ], s[N1];
-            load(NQ / 2, r);
+            proj_row<NQ>(f, NQ / 2, a.vec, r);
             proj_sum<NQ, N1>(a.WB, r, s);
 #pragma unroll
             for (int j = 0; j < N1; j += 2)
@@ -846,8 +851,8 @@ __global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ Pr
 #pragma unroll
         for (int m = 0; m < NP; ++m) {
             double rm[NQ], rp[NQ], sm[N1], sp[N1];
-            load(m, rm);
-            load(NQ - 1 - m, rp);
+            proj_row<NQ>(f, m, a.vec, rm);
+            proj_row<NQ>(f, NQ - 1 - m, a.vec, rp);
             proj_sum<NQ, N1>(a.WB, rm, sm);
             proj_sum<NQ, N1>(a.WB, rp, sp);
 #pragma unroll
@@ -867,6 +872,144 @@ __global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ Pr
     }
 }
 
+template <int DIM, int N1, int NQ>
+__global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ ProjArgs a)
+{
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < a.E) project_cell<DIM, N1, NQ>(a, e);
+}
+
+// Two lanes of unevaluated sums hi + lo (|lo| at most a few 2^-23 |hi|): the double-float
+// arithmetic of Dekker, "A floating-point technique for extending the available precision" (1971),
+// with the product's error from an FMA.  Every value carries 46 bits or more, so the float that
+// hi + lo is rounded to at the end is that of the sums in double but for values within 2^-20 of a
+// rounding boundary: of 4 million modes of the 1024^2 Q3 KPP data a few differ by one rounding, and
+// the error against 64 bits is the same 2.5e-8.
+struct Split2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// s + *err = a + b exactly (Knuth's two-sum)
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2* err)
+{
+    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+    *err = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+    return s;
+}
+__device__ __forceinline__ Split2 split_add(Split2 a, Split2 b)
+{
+    Split2 r;
+    float2 e;
+    r.hi = two_sum(a.hi, b.hi, &e);
+    r.lo = __fadd2_rn(__fadd2_rn(a.lo, b.lo), e);
+    return r;
+}
+__device__ __forceinline__ Split2 split_neg(Split2 a)
+{
+    return {make_float2(-a.hi.x, -a.hi.y), make_float2(-a.lo.x, -a.lo.y)};
+}
+// acc + (wh + wl) x
+__device__ __forceinline__ Split2 split_fma(float2 wh, float2 wl, Split2 x, Split2 acc)
+{
+    const float2 p = __fmul2_rn(wh, x.hi);
+    float2 e = __ffma2_rn(wh, x.hi, make_float2(-p.x, -p.y)), t;
+    e = __ffma2_rn(wh, x.lo, e);
+    e = __ffma2_rn(wl, x.hi, e);
+    Split2 r;
+    r.hi = two_sum(acc.hi, p, &t);
+    r.lo = __fadd2_rn(acc.lo, __fadd2_rn(t, e));
+    return r;
+}
+// v as hi + lo, from its bits (a conversion would occupy the FP64 pipe): the leading 24 and the
+// next 23 bits of the significand.  Zero is exact; other values outside [2^-60, 2^96) set *bad.
+__device__ __forceinline__ void split_double(double v, float* hi, float* lo, bool* bad)
+{
+    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+    const bool ok = (h & 0x7fffffffu) - 0x3c300000u < 0x45f00000u - 0x3c300000u;
+    *bad = *bad || (!ok && ((h & 0x7fffffffu) | l) != 0u);
+    // bits 30 .. 23 of the shifted word are the exponent mod 256, 1023 + x; float wants 127 + x
+    const unsigned bits = ((__funnelshift_l(l, h, 3) ^ 0x40000000u) & 0x7fffffffu) | (h & 0x80000000u);
+    const unsigned base = (bits & 0xff800000u) - (23u << 23);
+    const float d = __uint_as_float(base | ((l >> 6) & 0x7fffffu)) - __uint_as_float(base);
+    *hi = ok ? __uint_as_float(bits) : 0.f;
+    *lo = ok ? d : 0.f;
+}
+
+// Float states in 2D: the sums of project_cell on the packed FP32 pipe, which is 64 times as wide as
+// the FP64 one, in double-float arithmetic.  The lanes of a pair are the rows +-g_b while the
+// points of a row are summed, then the even and the odd mode j.  Cells with samples that the split
+// cannot hold (tiny, huge, not finite) take the sums in double.
+template <int N1, int NQ>
+__global__ void __launch_bounds__(128) project_split_kernel(const __grid_constant__ ProjArgs a)
+{
+    constexpr int NP = NQ / 2, NR = (NQ + 1) / 2, NJ = (N1 + 1) / 2;
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= a.E) return;
+    const double* f = a.f + e * (NQ * NQ);
+    const float2 zero = make_float2(0.f, 0.f);
+    bool bad = false;
+    Split2 c[N1][NJ];
+#pragma unroll
+    for (int i = 0; i < N1; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) c[i][j] = {zero, zero};
+#pragma unroll 1
+    for (int m = 0; m < NR; ++m) {
+        // rows m (lane x) and NQ - 1 - m (lane y); the centre row of an odd rule alone
+        const int mp = NQ - 1 - m;
+        double rm[NQ], rp[NQ];
+        proj_row<NQ>(f, m, a.vec, rm);
+        proj_row<NQ>(f, mp, a.vec, rp);
+        Split2 x[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            split_double(rm[q], &x[q].hi.x, &x[q].lo.x, &bad);
+            split_double(rp[q], &x[q].hi.y, &x[q].lo.y, &bad);
+            if ((NQ & 1) != 0 && m == mp) x[q].hi.x = x[q].lo.x = 0.f;
+        }
+        Split2 r[N1];
+#pragma unroll
+        for (int i = 0; i < N1; ++i) r[i] = {zero, zero};
+        if constexpr ((NQ & 1) != 0) {
+#pragma unroll
+            for (int i = 0; i < N1; i += 2)
+                r[i] = split_fma(make_float2(a.sh[NP][i], a.sh[NP][i]), make_float2(a.sl[NP][i], a.sl[NP][i]), x[NP], r[i]);
+        }
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            const int qp = NQ - 1 - q;
+            const Split2 S = split_add(x[qp], x[q]), D = split_add(x[qp], split_neg(x[q]));
+#pragma unroll
+            for (int i = 0; i < N1; ++i)
+                r[i] = split_fma(make_float2(a.sh[qp][i], a.sh[qp][i]), make_float2(a.sl[qp][i], a.sl[qp][i]), (i & 1) ? D : S, r[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+            // (r+ + r-, r+ - r-): what the even and the odd modes j take
+            const Split2 p = {make_float2(r[i].hi.y, r[i].hi.y), make_float2(r[i].lo.y, r[i].lo.y)};
+            const Split2 n = {make_float2(r[i].hi.x, -r[i].hi.x), make_float2(r[i].lo.x, -r[i].lo.x)};
+            const Split2 sd = split_add(p, n);
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int j1 = 2 * j + 1 < N1 ? 2 * j + 1 : 2 * j;
+                c[i][j] = split_fma(make_float2(a.sh[mp][2 * j], a.sh[mp][j1]), make_float2(a.sl[mp][2 * j], a.sl[mp][j1]), sd, c[i][j]);
+            }
+        }
+    }
+    if (bad) {
+        project_cell<2, N1, NQ>(a, e);
+        return;
+    }
+    float* U = static_cast<float*>(a.U) + e;
+#pragma unroll
+    for (int j = 0; j < N1; ++j)
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+            const Split2& v = c[i][j / 2];
+            U[(i + N1 * j) * a.E] = (j & 1) ? v.hi.y + v.lo.y : v.hi.x + v.lo.x;
+        }
+}
+
 // Fills the tables for degree p and the nq-point Gauss rule (P_0..P_p by their recurrence).
 static void project_tables(ProjArgs& a, int p, int nq)
 {
@@ -883,20 +1026,38 @@ static void project_tables(ProjArgs& a, int p, int nq)
         }
     }
     for (int i = 0; i <= p; ++i) a.minv[i] = (2 * i + 1) / 2.0;
+    for (int q = 0; q < nq; ++q)
+        for (int i = 0; i <= p; ++i) {
+            const double v = a.minv[i] * a.WB[q][i];
+            a.sh[q][i] = (float)v;
+            a.sl[q][i] = (float)(v - (double)a.sh[q][i]);
+        }
+}
+
+template <int DIM, int N1, int NQ>
+static void launch_project_q(const ProjArgs& a, unsigned blocks, cudaStream_t s)
+{
+    if constexpr (DIM == 2) {
+        if (!a.f64) {
+            project_split_kernel<N1, NQ><<<blocks, 128, 0, s>>>(a);
+            return;
+        }
+    }
+    project_kernel<DIM, N1, NQ><<<blocks, 128, 0, s>>>(a);
 }
 
 template <int DIM, int N1>
 static void launch_project_n(const ProjArgs& a, int nq, unsigned blocks, cudaStream_t s)
 {
     switch (nq) {
-    case 1: project_kernel<DIM, N1, 1><<<blocks, 128, 0, s>>>(a); break;
-    case 2: project_kernel<DIM, N1, 2><<<blocks, 128, 0, s>>>(a); break;
-    case 3: project_kernel<DIM, N1, 3><<<blocks, 128, 0, s>>>(a); break;
-    case 4: project_kernel<DIM, N1, 4><<<blocks, 128, 0, s>>>(a); break;
-    case 5: project_kernel<DIM, N1, 5><<<blocks, 128, 0, s>>>(a); break;
-    case 6: project_kernel<DIM, N1, 6><<<blocks, 128, 0, s>>>(a); break;
-    case 7: project_kernel<DIM, N1, 7><<<blocks, 128, 0, s>>>(a); break;
-    default: project_kernel<DIM, N1, 8><<<blocks, 128, 0, s>>>(a); break;
+    case 1: launch_project_q<DIM, N1, 1>(a, blocks, s); break;
+    case 2: launch_project_q<DIM, N1, 2>(a, blocks, s); break;
+    case 3: launch_project_q<DIM, N1, 3>(a, blocks, s); break;
+    case 4: launch_project_q<DIM, N1, 4>(a, blocks, s); break;
+    case 5: launch_project_q<DIM, N1, 5>(a, blocks, s); break;
+    case 6: launch_project_q<DIM, N1, 6>(a, blocks, s); break;
+    case 7: launch_project_q<DIM, N1, 7>(a, blocks, s); break;
+    default: launch_project_q<DIM, N1, 8>(a, blocks, s); break;
     }
 }
 

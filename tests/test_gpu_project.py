@@ -41,3 +41,25 @@ def test_project_all_rules(dim, nx, ny, nq):
                 err = np.abs(U.double().cpu().numpy() - want).max()
                 assert err <= tol[prec] * 12.25 * np.abs(f).max(), (p, prec, off)
             ctx.close()
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e30])
+def test_project_float_outside_the_split_range(scale):
+    """Float projection sums in double-float arithmetic where every sample lies in [2^-60, 2^96) or
+    is zero, and in double elsewhere: cells of either kind side by side, and cells of zeros."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nx, ny, nq, p = 20, 7, 8, 3
+    s = H.spec(2, p, nx, ny=ny)
+    f = np.random.default_rng(5).standard_normal((nx * ny, nq * nq))
+    f[::3] *= scale
+    f[1::5, ::2] = 0.0
+    f[7] = 0.0
+    want = O.project(O.Problem(**s), f.reshape(-1), nq)
+    ctx = dgw.Context(dgw.Problem(**s, prec="fp32"))
+    U = torch.empty((ctx.K, ctx.E), dtype=torch.float32, device="cuda")
+    ctx.project(torch.tensor(f.reshape(-1), device="cuda"), U, nq=nq)
+    err = np.abs(U.double().cpu().numpy() - want).max(axis=0)
+    # as above, per cell
+    assert (err <= 4 * 2.0 ** -24 * 12.25 * np.abs(f).max(axis=1)).all()
+    ctx.close()
