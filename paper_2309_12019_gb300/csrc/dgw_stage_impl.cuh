@@ -179,9 +179,7 @@ __device__ __forceinline__ double div_w(double a, double b) { return a * __drcp_
 // gamma of Eq. (sensor / gensensor) before the exponent q, min(1, r) with r = ||D|| / (W ||U||)
 // through the squares qd = ||D||^2, beta0 = ||U||^2 and W^2: one reciprocal square root in place
 // of two square roots and two divisions (double; the products stay in range while qd W^2 beta0
-// does, else the roots are taken one by one).  rr receives r (1 if not below 1).  With the integer
-// comparisons: rotation at 256^2 Q2, 149 -> 142 us a stage (tiles of 2 rows in place of 4, which
-// load the SMs more evenly there, 149).
+// does, else the roots are taken one by one).  rr receives r (1 if not below 1).
 __device__ __forceinline__ double sensor_ratio(double qd, double beta0, double W, double eps_s, double* rr)
 {
     const double W2 = W * W, den = W2 * beta0, pr = qd * den;
