@@ -122,9 +122,7 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
 
 // Volume term acc_i = sum_q W_q P_i'(g_q) F(U_h(g_q)) (acc_0 = 0) and lambda_e = max (|v| + c) over
 // the points, on the symmetric nodes.  Float with two node pairs (p = 2, 3): the pairs travel as
-// the lanes of packed FP32 instructions, which the issue-bound kernel needs fewer of.  With the
-// update of (rho, m) in pairs: Sod train of 2^22 cells, p = 2, 91.8 -> 86.8 us a stage (the 403 MB it
-// moves would take 60).
+// the lanes of packed FP32 instructions, which the issue-bound kernel needs fewer of.
 template <int P>
 __device__ __forceinline__ void euler_volume(const KParams& A, const Tab<P>& T, const Real (&c)[3][P + 1], bool need_lam,
                                              Real (&acc)[3][P + 1], Real& lam)
