@@ -24,9 +24,7 @@ constexpr int kTileX2 = 32;
 constexpr int kTileY2 = 4;
 constexpr int kBoxX2 = kTileX2 + 8;
 constexpr int stage_lanes(bool f64) { return f64 ? 1 : 2; }
-// (double: 2 rows; a stage is bound by the FP64 pipe of the busiest SM, and 512 tiles of 4 rows on
-// 152 SMs, 256^2 cells, leave some with four of them against 3.4 on average)
-constexpr int stage_thread_rows(bool f64) { return f64 ? kTileY2 / 2 : 2 * kTileY2; }
+constexpr int stage_thread_rows(bool f64) { return f64 ? kTileY2 : 2 * kTileY2; }
 constexpr int stage_rows(bool f64) { return stage_thread_rows(f64) * stage_lanes(f64); }
 // The persistent float stage kernel (whole-mesh launches): one CTA of 512 threads per SM
 // walks tiles of kTileX2 x kPRows cells; its boxes are kBoxX2 x (kPRows + 2) x K (Uk) and
