@@ -78,17 +78,15 @@ struct dgw_ctx {
     void* adj_b1 = nullptr;      // adjoint: lambda of stage 2
     void* adj_b2 = nullptr;      // adjoint: lambda of stage 1
     std::map<std::pair<const void*, int>, bool> no_tmap;
-    // dgw_rk_step_host pipeline: streams for input copies, output copies and a pool per
-    // stage; one event per (input copy or stage, band); the join events
-    cudaStream_t band_st[2 + 3 * 4] = {};
+    // dgw_rk_step_host pipeline: streams for input copies, output copies and each stage; one event per (input copy or stage, band); the join events
+    cudaStream_t band_st[2 + 3] = {};
     cudaEvent_t band_ev[4][16] = {};
     cudaEvent_t band_join[2] = {};
     std::map<BandKey, cudaGraphExec_t> band_graphs;   // null: replay not possible (direct launches)
 };
 
 static const int kBands = 16;
-static const int kStageStreams = 4;          // band kernels of one stage run concurrently
-static const int kBandStreams = 2 + 3 * kStageStreams;
+static const int kBandStreams = 2 + 3;
 
 static const int kMassBlocks = 1024;
 static const int kMassThreads = 256;
@@ -602,17 +600,18 @@ extern "C" dgw_status dgw_rk_step(dgw_ctx* c, void* U, double dt, int nsteps, vo
 }
 
 // One SSP-RK3 step of a 2D mesh that is not periodic in y, as a wavefront over bands of
-// tile rows: stage r of band b reads stage r - 1 on bands b - 1 .. b + 1 only, and bands of
-// one stage do not depend on each other.  So the input copy of a band, the three stages
-// and the output copy of a finished band overlap, and band kernels of a stage run
-// concurrently.  Streams: input copies (in order), output copies (in order), and a pool
-// of kStageStreams per stage (band b on stream b mod kStageStreams); one event per (input
-// copy or stage, band); all joined to the caller's stream s at both ends.  copy_in: U_in
-// (host) is copied to c->Uhost_dev band by band first; copy_out: the result is copied to
-// U_out band by band.  Stage 3 writes U in place; the old U of band b is still read by
-// stage 1 of bands b - 1 and b + 1 (halo rows) and by stages 2, 3 of band b (own rows):
-// stage 3 of band b waits for stage 2 of bands b - 1 .. b + 1, which waited for stage 1
-// of bands b - 2 .. b + 2.
+// tile rows: stage r of band b reads stage r - 1 only on bands b - 1 .. b + 1.  So the input
+// copy of a band, the three stages and the output copy of a finished band overlap.  Streams,
+// each in the order of the bands: input copies, output copies, one per stage; one event per
+// (input copy or stage, band); all joined to the caller's stream s at both ends.  As a stream
+// keeps its order, a stage waits for the highest band that it reads alone.  (A pool of four
+// streams per stage, each kernel waiting for three bands, was as fast replayed from a graph, 0.64
+// ms for 1024^2 Q3; launched directly, as on the default stream, its 276 calls took 0.80 ms, these
+// 0.67.)  copy_in: U_in (host) is copied to c->Uhost_dev band by band first; copy_out:
+// the result is copied to U_out band by band.  Stage 3 writes U in place; the old U of band b is
+// still read by stage 1 of bands b - 1 and b + 1 (halo rows) and by stages 2, 3 of band b (own
+// rows): stage 3 of band b waits for stage 2 of the bands up to b + 1, which waited for stage 1
+// of the bands up to b + 2.
 static dgw_status banded_step(dgw_ctx* c, const void* U_in, void* U_out, double dt, bool copy_in,
                               bool copy_out, cudaStream_t s)
 {
@@ -621,7 +620,6 @@ static dgw_status banded_step(dgw_ctx* c, const void* U_in, void* U_out, double 
     const int nb = trows < kBands ? trows : kBands;
     cudaStream_t* st = c->band_st;
     cudaStream_t in_st = st[0], out_st = st[1];
-    auto stage_st = [&](int r, int b) { return st[2 + r * kStageStreams + b % kStageStreams]; };
     auto& ev = c->band_ev;
     DGW_CUDA(cudaEventRecord(c->band_join[0], s));
     for (int i = 0; i < kBandStreams; ++i) DGW_CUDA(cudaStreamWaitEvent(st[i], c->band_join[0], 0));
@@ -650,14 +648,8 @@ static dgw_status banded_step(dgw_ctx* c, const void* U_in, void* U_out, double 
         if (r == 1) { a.Uk = c->S1; a.Un = U; a.Uout = c->S2; a.cn = 0.75; a.ck = 0.25; a.cl = 0.25 * dt; }
         if (r == 2) { a.Uk = c->S2; a.Un = U; a.Uout = U; a.cn = 1.0 / 3.0; a.ck = 2.0 / 3.0; a.cl = 2.0 / 3.0 * dt; }
         for (int b = 0; b < nb; ++b) {
-            cudaStream_t ks = stage_st(r, b);
-            if (r == 0) {
-                // the input copies complete in order: the highest band read suffices
-                if (copy_in) DGW_CUDA(cudaStreamWaitEvent(ks, ev[0][b + 1 < nb ? b + 1 : nb - 1], 0));
-            } else {
-                for (int d = b - 1; d <= b + 1; ++d)
-                    if (d >= 0 && d < nb) DGW_CUDA(cudaStreamWaitEvent(ks, ev[r][d], 0));
-            }
+            cudaStream_t ks = st[2 + r];
+            if (r > 0 || copy_in) DGW_CUDA(cudaStreamWaitEvent(ks, ev[r][b + 1 < nb ? b + 1 : nb - 1], 0));
             a.tile_row0 = t0[b];
             a.tile_rows = t0[b + 1] - t0[b];
             DGW_CUDA(launch(c, a, 0, ks));
@@ -677,7 +669,7 @@ static dgw_status banded_step(dgw_ctx* c, const void* U_in, void* U_out, double 
         DGW_CUDA(cudaEventRecord(c->band_join[1], out_st));
         DGW_CUDA(cudaStreamWaitEvent(s, c->band_join[1], 0));
     } else {
-        for (int b = 0; b < nb; ++b) DGW_CUDA(cudaStreamWaitEvent(s, ev[3][b], 0));
+        DGW_CUDA(cudaStreamWaitEvent(s, ev[3][nb - 1], 0));
     }
     return DGW_OK;
 }
