@@ -120,11 +120,93 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
     return g;
 }
 
+// Volume term acc_i = sum_q W_q P_i'(g_q) F(U_h(g_q)) (acc_0 = 0) and lambda_e = max (|v| + c) over
+// the points, on the symmetric nodes.  Float with two node pairs (p = 2, 3): the pairs travel as
+// the lanes of packed FP32 instructions, which the issue-bound kernel needs fewer of.  With the
+// update of (rho, m) in pairs: Sod train of 2^22 cells, p = 2, 91.8 -> 86.8 us a stage (the 403 MB it
+// moves would take 60).
+template <int P>
+__device__ __forceinline__ void euler_volume(const KParams& A, const Tab<P>& T, const Real (&c)[3][P + 1], bool need_lam,
+                                             Real (&acc)[3][P + 1], Real& lam)
+{
+    constexpr int N1 = P + 1, NQ = P + 2;
+    if constexpr (kF32 && P >= 2) {
+        auto two = [](Real x) { return make_float2((float)x, (float)x); };
+        // table entry i of the two positive nodes, outermost first
+        auto pairB = [&](int i) { return make_float2((float)T.B[NQ - 1][i], (float)T.B[NQ - 2][i]); };
+        float2 up[3], um[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float2 e = __ffma2_rn(pairB(2), two(c[q][2]), two(c[q][0]));
+            float2 o = __fmul2_rn(pairB(1), two(c[q][1]));
+            if constexpr (P == 3) o = __ffma2_rn(pairB(3), two(c[q][3]), o);
+            up[q] = __fadd2_rn(e, o);
+            um[q] = vsub(e, o);
+        }
+        // F_2, F_3 and |v| + c at both lanes of (rho, m, rho E)
+        auto point = [&](const float2 (&u)[3], float2 (&F)[3]) {
+            const float2 inv = make_float2(rcp_e(u[0].x), rcp_e(u[0].y));
+            const float2 v = __fmul2_rn(u[1], inv);
+            const float2 pr = __fmul2_rn(two(A.gm1), __ffma2_rn(__fmul2_rn(two(Real(-0.5)), u[1]), v, u[2]));
+            F[0] = u[1];
+            F[1] = __ffma2_rn(u[1], v, pr);
+            F[2] = __fmul2_rn(__fadd2_rn(u[2], pr), v);
+            if (need_lam) {
+                const float2 s = __fmul2_rn(__fmul2_rn(two(A.gam), pr), inv);
+                lam = max_nan(lam, max_nan(fabsf(v.x) + sqrt_e(s.x), fabsf(v.y) + sqrt_e(s.y)));
+            }
+        };
+        float2 Fp[3], Fm[3];
+        point(up, Fp);
+        point(um, Fm);
+        Real Fc[3] = {Real(0), Real(0), Real(0)};
+        if constexpr (P == 3) {       // the centre node
+            constexpr int qc = NQ / 2;
+            Real u[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) u[q] = fma(T.B[qc][2], c[q][2], c[q][0]);
+            const EulerState st = euler_prim(A, u[0], u[1], u[2]);
+            euler_flux(st, u[1], u[2], Fc);
+            if (need_lam) lam = max_nan(lam, euler_speed(A, st));
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float2 S = __fadd2_rn(Fp[q], Fm[q]), D = vsub(Fp[q], Fm[q]);
+            acc[q][0] = Real(0);
+#pragma unroll
+            for (int i = 1; i < N1; ++i) {
+                const float2 f = (i & 1) ? S : D;        // P_i' is even for odd i
+                Real t = fma(T.WD[NQ - 2][i], f.y, T.WD[NQ - 1][i] * f.x);
+                if (P == 3 && (i & 1)) t = fma(T.WD[NQ / 2][i], Fc[q], t);
+                acc[q][i] = t;
+            }
+        }
+    } else {
+        Real u[3][NQ], F[3][NQ];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) interp_sym<N1, NQ>(T.B, c[q], u[q]);
+#pragma unroll
+        for (int g = 0; g < NQ; ++g) {
+            const EulerState st = euler_prim(A, u[0][g], u[1][g], u[2][g]);
+            Real f[3];
+            euler_flux(st, u[1][g], u[2][g], f);
+            if (need_lam) lam = max_nan(lam, euler_speed(A, st));
+#pragma unroll
+            for (int q = 0; q < 3; ++q) F[q][g] = f[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            project_sym<true, N1, NQ>(T.WD, F[q], acc[q]);
+            acc[q][0] = Real(0);
+        }
+    }
+}
+
 // MODE 0: stage / residual; MODE 1: sensor only (writes gamma_out).
 template <int P, int MODE>
 __global__ void __launch_bounds__(TX, kF32 ? 8 : 4) euler_kernel(const __grid_constant__ KParams A)
 {
-    constexpr int N1 = P + 1, NQ = P + 2;
+    constexpr int N1 = P + 1;
     __shared__ EulerSmem<P> S;
     pdl_begin();
     const Tab<P>& T = tab<P>();
@@ -209,33 +291,9 @@ __global__ void __launch_bounds__(TX, kF32 ? 8 : 4) euler_kernel(const __grid_co
 
     // ---- 1b. volume term: acc_i = sum_q W_q P_i'(g_q) F(U_h(g_q)); lambda_e ----
     Real acc[3][N1];
-#pragma unroll
-    for (int comp = 0; comp < 3; ++comp)
-#pragma unroll
-        for (int k = 0; k < N1; ++k) acc[comp][k] = Real(0);
     Real lam = Real(0);
     const bool need_lam = A.stab != STAB_DG && !A.lam_fixed;
-    if (in) {
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            Real u[3];
-#pragma unroll
-            for (int comp = 0; comp < 3; ++comp) {
-                Real s = Real(0);
-#pragma unroll
-                for (int k = 0; k < N1; ++k) s = fma(T.B[q][k], c[comp][k], s);
-                u[comp] = s;
-            }
-            const EulerState st = euler_prim(A, u[0], u[1], u[2]);
-            Real F[3];
-            euler_flux(st, u[1], u[2], F);
-            if (need_lam) lam = max_nan(lam, euler_speed(A, st));
-#pragma unroll
-            for (int comp = 0; comp < 3; ++comp)
-#pragma unroll
-                for (int k = 0; k < N1; ++k) acc[comp][k] = fma(T.WD[q][k], F[comp], acc[comp][k]);
-        }
-    }
+    if (in) euler_volume<P>(A, T, c, need_lam, acc, lam);
 
     // ---- 2. faces f = 0 .. nt of the tile ----
     for (int f = tid; f <= nt; f += TX) {
@@ -274,29 +332,41 @@ __global__ void __launch_bounds__(TX, kF32 ? 8 : 4) euler_kernel(const __grid_co
     // lambda_e: also |v| + c at the cell's two ends, its own states at faces tid, tid + 1
     if (need_lam) lam = max_nan(lam, max_nan(S.sp[1][tid], S.sp[0][tid + 1]));
     const Real ngs = A.stab == STAB_DG ? Real(0) : -(gamma * (A.lam_fixed ? A.lambda_nu : lam) * Real(1.0 / P));
+    // (rho, m) of a mode as a pair (packed in float), rho E by itself
+    using E2 = std::conditional_t<kF32, float2, double2>;
+    auto pair = [](Real x, Real y) { E2 v; v.x = x; v.y = y; return v; };
+    auto update = [&](auto hm, auto hp, auto acc_k, int k, const auto* cc, auto un_k) {
+        // -P_k(+1) H_right + P_k(-1) H_left
+        auto r = (k & 1) ? vsub(acc_k, vadd(hm, hp)) : vadd(acc_k, vsub(hm, hp));
+        if (k > 0) {
+            auto kc = vmul(T.A1[k][k], cc[k]);
+#pragma unroll
+            for (int m = 1; m < N1; ++m)
+                if (m != k && ((k + m) & 1) == 0) kc = vfma(vbc<decltype(kc)>(T.A1[k][m]), cc[m], kc);
+            r = vfma(vbc<decltype(r)>(ngs), kc, r);
+        }
+        auto out = vfma(vbc<decltype(r)>(A.cl), vmul(A.two_h * T.minv[k], r), vmul(A.ck, cc[k]));
+        if (A.has_un) out = vfma(vbc<decltype(r)>(A.cn), un_k, out);
+        return out;
+    };
+    E2 c2[N1];
+#pragma unroll
+    for (int k = 0; k < N1; ++k) c2[k] = pair(c[0][k], c[1][k]);
+    const E2 hm2 = pair(S.hf[0][tid], S.hf[1][tid]), hp2 = pair(S.hf[0][tid + 1], S.hf[1][tid + 1]);
+    const Real hm3 = S.hf[2][tid], hp3 = S.hf[2][tid + 1];
+    E2 chk2 = pair(Real(0), Real(0));
     Real chk = Real(0);
 #pragma unroll
-    for (int comp = 0; comp < 3; ++comp) {
-        const Real hm = S.hf[comp][tid], hp = S.hf[comp][tid + 1];
-#pragma unroll
-        for (int k = 0; k < N1; ++k) {
-            // -P_k(+1) H_right + P_k(-1) H_left
-            Real r = acc[comp][k] + ((k & 1) ? -(hm + hp) : (hm - hp));
-            if (k > 0) {
-                Real kc = Real(0);
-#pragma unroll
-                for (int m = 1; m < N1; ++m)
-                    if (((k + m) & 1) == 0) kc = fma(T.A1[k][m], c[comp][m], kc);
-                r = fma(ngs, kc, r);
-            }
-            const Real Lk = (A.two_h * T.minv[k]) * r;
-            const int64_t idx = (int64_t)(comp * N1 + k) * E + gx;
-            Real out = fma(A.cl, Lk, A.ck * c[comp][k]);
-            if (A.has_un) out = fma(A.cn, un[comp][k], out);
-            chk = fma(out, Real(0), chk);
-            A.Uout[idx] = out;
-        }
+    for (int k = 0; k < N1; ++k) {
+        const E2 o2 = update(hm2, hp2, pair(acc[0][k], acc[1][k]), k, c2, pair(un[0][k], un[1][k]));
+        const Real o3 = update(hm3, hp3, acc[2][k], k, c[2], un[2][k]);
+        chk2 = vfma(o2, pair(Real(0), Real(0)), chk2);
+        chk = fma(o3, Real(0), chk);
+        A.Uout[(int64_t)k * E + gx] = o2.x;
+        A.Uout[(int64_t)(N1 + k) * E + gx] = o2.y;
+        A.Uout[(int64_t)(2 * N1 + k) * E + gx] = o3;
     }
+    chk += chk2.x + chk2.y;
     if (chk != chk) atomicOr(A.flag, 1u);
 }
 
