@@ -376,11 +376,6 @@ __global__ void __launch_bounds__(kLineThreads) line_euler_kernel(const __grid_c
 // Eight lanes per cell (double)
 // ------------------------------------------------------------------------------------
 __device__ __forceinline__ Real group_get(Real v, int src) { return __shfl_sync(0xffffffffu, v, src, 8); }
-// Numbers >= 0 are ordered like their bits, and a comparison of integers stays off the FP64 pipe.
-__device__ __forceinline__ long long bits_of(double v) { return __double_as_longlong(v); }
-__device__ __forceinline__ long long bits_of(float v) { return __float_as_int(v); }
-__device__ __forceinline__ bool less_pos(Real a, Real b) { return bits_of(a) < bits_of(b); }
-__device__ __forceinline__ Real max_pos(Real a, Real b) { return less_pos(a, b) ? b : a; }
 __device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 __device__ __forceinline__ bool not_finite(float v) { return (__float_as_int(v) & 0x7f800000) == 0x7f800000; }
 // largest v >= 0 of the cell's lanes

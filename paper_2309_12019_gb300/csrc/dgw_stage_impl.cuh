@@ -163,10 +163,40 @@ __device__ __forceinline__ void sincos_r(double x, double* s, double* c) { sinco
 __device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
 __device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
 
+// Comparisons of numbers >= 0.  In double as integers (such numbers are ordered like their bits):
+// a double comparison or maximum occupies the FP64 pipe like a product and its result takes about
+// 180 cycles, that of an integer one a few.
+__device__ __forceinline__ bool less_pos(float a, float b) { return a < b; }
+__device__ __forceinline__ bool less_pos(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+__device__ __forceinline__ float max_pos(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_pos(double a, double b) { return less_pos(a, b) ? b : a; }
+
 // a / b for the sensor weights: the hardware reciprocal in float (at most 2 ulp; the
 // divisors here lie in [1e-12, 1e30]), the correctly rounded quotient in double.
 __device__ __forceinline__ float div_w(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double div_w(double a, double b) { return a / b; }
+__device__ __forceinline__ double div_w(double a, double b) { return a * __drcp_rn(b); }
+
+// gamma of Eq. (sensor / gensensor) before the exponent q, min(1, r) with r = ||D|| / (W ||U||)
+// through the squares qd = ||D||^2, beta0 = ||U||^2 and W^2: one reciprocal square root in place
+// of two square roots and two divisions (double; the products stay in range while qd W^2 beta0
+// does, else the roots are taken one by one).  rr receives r (1 if not below 1).  With the integer
+// comparisons: rotation at 256^2 Q2, 149 -> 142 us a stage (tiles of 2 rows in place of 4, which
+// load the SMs more evenly there, 149).
+__device__ __forceinline__ double sensor_ratio(double qd, double beta0, double W, double eps_s, double* rr)
+{
+    const double W2 = W * W, den = W2 * beta0, pr = qd * den;
+    *rr = 1.0;
+    if (!less_pos(1e-280, pr) || !less_pos(pr, 1e280) || !less_pos(1e-140, W2) || !less_pos(W2, 1e140)) {
+        const double num = sqrt(fmax(qd, 0.0)) / W;
+        if (num <= eps_s) return 0.0;
+        if (beta0 <= 0.0) return 1.0;
+        *rr = num / sqrt(beta0);
+    } else {
+        if (!less_pos((eps_s * eps_s) * W2, qd)) return 0.0;
+        if (less_pos(qd, den)) *rr = qd * rsqrt(pr);
+    }
+    return *rr < 1.0 ? *rr : 1.0;
+}
 
 constexpr double kPi = 3.14159265358979323846;
 
@@ -265,7 +295,7 @@ __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ Real vsub(Real a, Real b) { return a - b; }
 // a - b as one fused step: b * (-1) + a rounds once, exactly like the subtraction
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ Real vmax(Real a, Real b) { return fmax(a, b); }
+__device__ __forceinline__ Real vmax(Real a, Real b) { return max_pos(a, b); }   // of keys (>= 0)
 __device__ __forceinline__ float2 vmax(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 
 template <class V> struct Lanes { static constexpr int n = 1; };
@@ -408,7 +438,7 @@ __device__ __forceinline__ Real llf(const KParams& A, int axis, Real uL, Real uR
         return fma_x(mul_x(Real(-0.5), fabs(v)), uR - uL, mul_x(mul_x(Real(0.5), v), uL + uR));
     } else if (FLUX == FLUX_BURGERS) {
         const Real an = axis == 0 ? A.a0 : A.a1;
-        const Real s = mul_x(fabs(an), fmax(fabs(uL), fabs(uR)));
+        const Real s = mul_x(fabs(an), max_pos(fabs(uL), fabs(uR)));
         return fma_x(mul_x(Real(-0.5), s), uR - uL, mul_x(mul_x(Real(0.25), an), fma_x(uL, uL, mul_x(uR, uR))));
     } else {
         // x-normal: n.F = sin u, |F'.n| = |cos u| (maximal at multiples of pi);
@@ -746,9 +776,9 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     if (MODE == 0) {
 #pragma unroll
         for (int t = 0; t < TN; ++t) {
-            V xm = vbc<V>(0), xp = vbc<V>(0), ym = vbc<V>(0), yp = vbc<V>(0);
+            V xm = DIM == 1 ? c[0] : c[N1 * t], xp = xm, ym = c[t], yp = ym;
 #pragma unroll
-            for (int n = 0; n < N1; ++n) {
+            for (int n = 1; n < N1; ++n) {
                 const V kx = DIM == 1 ? c[n] : c[n + N1 * t];
                 xp = vadd(xp, kx);
                 xm = (n & 1) ? vsub(xm, kx) : vadd(xm, kx);
@@ -861,8 +891,10 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             for (int k = 1; k < K; ++k) dacc[k] = vfma(wl, vsub(c[k], cl[k]), dacc[k]);
         }
         V inv;
+        if (kF32 || A.stab == STAB_ZHAO) {
 #pragma unroll
-        for (int l = 0; l < L; ++l) lane(inv, l) = div_w(Real(1), lane(wsum, l));
+            for (int l = 0; l < L; ++l) lane(inv, l) = div_w(Real(1), lane(wsum, l));
+        }
         if (A.stab == STAB_ZHAO) {
             // the comparison sensor of Zhao et al. restated in Sec. 5.6: deviation of the
             // nonlinear weights from the linear ones, over its largest possible value (all
@@ -888,10 +920,20 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             }
         } else {
             // U - U* = sum_l w_l (c - c_l)
+            if constexpr (kF32) {
 #pragma unroll
-            for (int k = 1; k < K; ++k) dacc[k] = vmul(dacc[k], inv);
+                for (int k = 1; k < K; ++k) dacc[k] = vmul(dacc[k], inv);
+            }
             dacc[0] = vbc<V>(0);
             const V qd = qform<P>(T, dacc);
+            if constexpr (!kF32) {
+                Real r;
+                Real g = sensor_ratio(qd, beta0, wsum, A.eps_s, &r);
+                if (!A.q_one) g = pow(g, A.q);
+                if (less_pos(r, A.b)) g = Real(0);
+                gamma = g;
+                if (MODE == 1 && in[0]) A.gamma_out[(int64_t)gy[0] * A.nx + gx] = (double)g;
+            } else
 #pragma unroll
             for (int l = 0; l < L; ++l) {
                 const Real num = sqrt_r(fmax(lane(qd, l), Real(0)));
@@ -1099,8 +1141,8 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                 if (need_lam) {
 #pragma unroll
                     for (int l = 0; l < L; ++l) {   // |F'| = 1 in 2D; 1D: |cos u| (no shift)
-                        lane(lm, l) = fmax(lane(lm, l), speed_key<FLUX>(A, lane(uL, l), Real(0), Real(0)));
-                        lane(lp, l) = fmax(lane(lp, l), speed_key<FLUX>(A, lane(uR, l), Real(0), Real(0)));
+                        lane(lm, l) = max_pos(lane(lm, l), speed_key<FLUX>(A, lane(uL, l), Real(0), Real(0)));
+                        lane(lp, l) = max_pos(lane(lp, l), speed_key<FLUX>(A, lane(uR, l), Real(0), Real(0)));
                     }
                 }
                 Hq[q] = llf_kpp(uL, uR);
@@ -1128,8 +1170,8 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                         ur = (A.bc[bside] == BC_INFLOW_ZERO && dflux_axis<FLUX>(A, axis, ul, x, y) < Real(0)) ? Real(0) : ul;
                     }
                     if (need_lam) {
-                        lane(lm, l) = fmax(lane(lm, l), speed_key<FLUX>(A, ul, x, y));
-                        lane(lp, l) = fmax(lane(lp, l), speed_key<FLUX>(A, ur, x, y));
+                        lane(lm, l) = max_pos(lane(lm, l), speed_key<FLUX>(A, ul, x, y));
+                        lane(lp, l) = max_pos(lane(lp, l), speed_key<FLUX>(A, ur, x, y));
                     }
                     lane(Hq[q], l) = llf<FLUX>(A, axis, ul, ur, x, y);
                 }
@@ -1207,7 +1249,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     if (find_lam) {
 #pragma unroll
         for (int l = 0; l < L; ++l)
-            lane(lam, l) = speed_of_key<FLUX>(A, need_lam ? fmax(lane(lam, l), lam_s[cy[l]][lx]) : lane(lam, l));
+            lane(lam, l) = speed_of_key<FLUX>(A, need_lam ? max_pos(lane(lam, l), lam_s[cy[l]][lx]) : lane(lam, l));
     }
 
     // stabilization (Sec. 3), M^{-1}, RK combination (Eq. ssp)
@@ -1281,7 +1323,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
 }
 
 template <int P, int FLUX, int MODE>
-__global__ void __launch_bounds__(NTS, LS == 2 ? 512 / NTS : (kF32 ? 6 : 3)) stage_kernel(const __grid_constant__ KParams A)
+__global__ void __launch_bounds__(NTS, LS == 2 ? 512 / NTS : (kF32 ? 6 : 384 / NTS)) stage_kernel(const __grid_constant__ KParams A)
 {
     pdl_begin();
     extern __shared__ __align__(128) unsigned char smem_raw[];
