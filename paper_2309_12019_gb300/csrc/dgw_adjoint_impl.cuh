@@ -68,6 +68,24 @@ __device__ __forceinline__ Real dspeed(const KParams& A, Real u)
     return an * (u > Real(0) ? Real(1) : (u < Real(0) ? Real(-1) : Real(0)));
 }
 
+// g[q] = sum_i r[i] P_i'(g_q) on the symmetric nodes (P_i' has the parity of i - 1)
+template <int N1, int NQ>
+__device__ __forceinline__ void deriv_sym(const Real (&D)[NQ][N1], const Real (&r)[N1], Real (&g)[NQ])
+{
+#pragma unroll
+    for (int m = 0; m < (NQ + 1) / 2; ++m) {
+        const int qp = NQ - 1 - m;
+        Real e = r[1], o = Real(0);            // P_1' = 1
+#pragma unroll
+        for (int i = 2; i < N1; ++i) {
+            if (i & 1) e = fma(D[qp][i], r[i], e);
+            else o = fma(D[qp][i], r[i], o);
+        }
+        g[qp] = e + o;
+        g[m] = e - o;
+    }
+}
+
 template <int P, int FLUX>
 __global__ void __launch_bounds__(128, P <= 2 ? 4 : 1) vjp_kernel(const KParams A, const Real* __restrict__ lam,
                                                   Real* __restrict__ wself, Real* __restrict__ wnb)
@@ -127,50 +145,44 @@ __global__ void __launch_bounds__(128, P <= 2 ? 4 : 1) vjp_kernel(const KParams 
             }
         }
     } else {
-        Real tc[N1][NQ], tvd[N1][NQ], tvb[N1][NQ];
-#pragma unroll
-        for (int j = 0; j < N1; ++j)
-#pragma unroll
-            for (int qa = 0; qa < NQ; ++qa) {
-                Real s0 = Real(0), s1 = Real(0), s2 = Real(0);
-#pragma unroll
-                for (int i = 0; i < N1; ++i) {
-                    s0 = fma(c[i + N1 * j], T.B[qa][i], s0);
-                    s1 = fma(v[i + N1 * j], T.D[qa][i], s1);
-                    s2 = fma(v[i + N1 * j], T.B[qa][i], s2);
-                }
-                tc[j][qa] = s0;
-                tvd[j][qa] = s1;
-                tvb[j][qa] = s2;
-            }
-#pragma unroll
+        // one Gauss row at a time, as the forward kernel: U_h and the gradient of lam reduced to the
+        // row, their values at its points on the symmetric nodes, F'(u).grad there, projected back.
+        // The rolled loop keeps one copy of the row's code: instruction fetch was the second largest
+        // stall of the kernel with the rows unrolled (gradient of 8 steps, 512^2 Q2, 2.77 -> 2.72 ms).
+#pragma unroll 1
         for (int qb = 0; qb < NQ; ++qb) {
-            Real row[N1];
+            Real rc[N1], rv[N1], rd[N1];
 #pragma unroll
-            for (int i = 0; i < N1; ++i) row[i] = Real(0);
+            for (int i = 0; i < N1; ++i) {
+                Real s0 = c[i], s1 = v[i], s2 = Real(0);
+#pragma unroll
+                for (int j = 1; j < N1; ++j) {
+                    s0 = fma(T.B[qb][j], c[i + N1 * j], s0);
+                    s1 = fma(T.B[qb][j], v[i + N1 * j], s1);
+                    s2 = fma(T.D[qb][j], v[i + N1 * j], s2);
+                }
+                rc[i] = s0;
+                rv[i] = s1;
+                rd[i] = s2;
+            }
+            Real u[NQ], gx[NQ], gy[NQ], row[N1];
+            interp_sym<N1, NQ>(T.B, rc, u);
+            interp_sym<N1, NQ>(T.B, rd, gy);
+            deriv_sym<N1, NQ>(T.D, rv, gx);
 #pragma unroll
             for (int qa = 0; qa < NQ; ++qa) {
-                Real u = Real(0), gx = Real(0), gy = Real(0);
-#pragma unroll
-                for (int j = 0; j < N1; ++j) {
-                    u = fma(tc[j][qa], T.B[qb][j], u);
-                    gx = fma(tvd[j][qa], T.B[qb][j], gx);
-                    gy = fma(tvb[j][qa], T.D[qb][j], gy);
-                }
-                const Real fx = FLUX == FLUX_ADVECT ? A.a0 : A.a0 * u;
-                const Real fy = FLUX == FLUX_ADVECT ? A.a1 : A.a1 * u;
-                const Real s = T.w[qa] * T.w[qb] * (fx * gx + fy * gy);
-#pragma unroll
-                for (int i = 0; i < N1; ++i) row[i] = fma(T.B[qa][i], s, row[i]);
                 if (need_lam) {
-                    const Real key = FLUX == FLUX_ADVECT ? Real(0) : fabs(u);
-                    if (key > kmax) { kmax = key; u_at = u; at_code = qa * 16 + qb; }
+                    const Real key = FLUX == FLUX_ADVECT ? Real(0) : fabs(u[qa]);
+                    if (key > kmax) { kmax = key; u_at = u[qa]; at_code = qa * 16 + qb; }
                 }
+                const Real g = fma(A.a0, gx[qa], A.a1 * gy[qa]);
+                u[qa] = FLUX == FLUX_ADVECT ? g : u[qa] * g;
             }
+            project_sym<false, N1, NQ>(T.WB, u, row);
 #pragma unroll
             for (int j = 0; j < N1; ++j)
 #pragma unroll
-                for (int i = 0; i < N1; ++i) ws[i + N1 * j] = fma(T.B[qb][j], row[i], ws[i + N1 * j]);
+                for (int i = 0; i < N1; ++i) ws[i + N1 * j] = fma(T.WB[qb][j], row[i], ws[i + N1 * j]);
         }
     }
 
@@ -205,34 +217,30 @@ __global__ void __launch_bounds__(128, P <= 2 ? 4 : 1) vjp_kernel(const KParams 
             tv[t] = sv;
         }
         Real eo[TN], en[TN];
-#pragma unroll
-        for (int t = 0; t < TN; ++t) { eo[t] = Real(0); en[t] = Real(0); }
+        Real uo[NFQ], un[NFQ], av[NFQ];
+        if constexpr (DIM == 1) {
+            uo[0] = to[0]; un[0] = tn[0]; av[0] = tv[0];
+        } else {
+            interp_sym<N1, NQ>(T.B, to, uo);
+            interp_sym<N1, NQ>(T.B, tn, un);
+            interp_sym<N1, NQ>(T.B, tv, av);
+        }
 #pragma unroll
         for (int q = 0; q < NFQ; ++q) {
-            Real uo = Real(0), un = Real(0), a = Real(0);
-            if (DIM == 1) { uo = to[0]; un = tn[0]; a = tv[0]; }
-            else {
-#pragma unroll
-                for (int t = 0; t < TN; ++t) {
-                    uo = fma(to[t], T.B[q][t], uo);
-                    un = fma(tn[t], T.B[q][t], un);
-                    a = fma(tv[t], T.B[q][t], a);
-                }
-                a *= T.w[q];
+            if (need_lam) {
+                const Real key = FLUX == FLUX_ADVECT ? Real(0) : fabs(uo[q]);
+                if (key > kmax) { kmax = key; u_at = uo[q]; at_code = 256 + f * 16 + q; }
             }
             Real ho, hn;
-            llf_grad<FLUX>(A, axis, sgn, uo, un, ho, hn);
-            const Real go = -a * ho, gn = -a * hn;
-#pragma unroll
-            for (int t = 0; t < TN; ++t) {
-                const Real bt = DIM == 1 ? Real(1) : T.B[q][t];
-                eo[t] = fma(go, bt, eo[t]);
-                en[t] = fma(gn, bt, en[t]);
-            }
-            if (need_lam) {
-                const Real key = FLUX == FLUX_ADVECT ? Real(0) : fabs(uo);
-                if (key > kmax) { kmax = key; u_at = uo; at_code = 256 + f * 16 + q; }
-            }
+            llf_grad<FLUX>(A, axis, sgn, uo[q], un[q], ho, hn);
+            uo[q] = -av[q] * ho;
+            un[q] = -av[q] * hn;
+        }
+        if constexpr (DIM == 1) {
+            eo[0] = uo[0]; en[0] = un[0];
+        } else {
+            project_sym<false, N1, NQ>(T.WB, uo, eo);
+            project_sym<false, N1, NQ>(T.WB, un, en);
         }
 #pragma unroll
         for (int t = 0; t < TN; ++t)
