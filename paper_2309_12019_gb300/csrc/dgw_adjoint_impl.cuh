@@ -459,15 +459,35 @@ __global__ void __launch_bounds__(128) gather_kernel(const int64_t E, const int 
         if (DIM == 2) jy = jy < 0 ? ny - 1 : (jy >= ny ? 0 : jy);
         nb[f] = (int64_t)jy * nx + jx;
     }
+    // the loads of up to eight modes are issued together: the kernel waits for memory (L2) and for
+    // nothing else (with the misfit's table: gradient of 8 steps, 512^2 Q2, 2.72 -> 2.58 ms)
+    constexpr int G = K < 8 ? K : 8;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        Real g = wself[k * E + e];
+    for (int k0 = 0; k0 < K; k0 += G) {
+        Real w[G][NF + 1], x[G][3];
 #pragma unroll
-        for (int f = 0; f < NF; ++f) g += wnb[((int64_t)(f ^ 1) * K + k) * E + nb[f]];
-        Real o = cv * g;
-        if (x0) o = fma(c0, x0[k * E + e], o);
-        if (x1) o = fma(c1, x1[k * E + e], o);
-        if (x2) o = fma(c2, x2[k * E + e], o);
-        out[k * E + e] = o;
+        for (int i = 0; i < G; ++i) {
+            const int k = k0 + i;
+            if (k >= K) continue;
+            w[i][NF] = wself[k * E + e];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) w[i][f] = wnb[((int64_t)(f ^ 1) * K + k) * E + nb[f]];
+            x[i][0] = x0 ? x0[k * E + e] : Real(0);
+            x[i][1] = x1 ? x1[k * E + e] : Real(0);
+            x[i][2] = x2 ? x2[k * E + e] : Real(0);
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const int k = k0 + i;
+            if (k >= K) continue;
+            Real g = w[i][NF];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) g += w[i][f];
+            Real o = cv * g;
+            if (x0) o = fma(c0, x[i][0], o);
+            if (x1) o = fma(c1, x[i][1], o);
+            if (x2) o = fma(c2, x[i][2], o);
+            out[k * E + e] = o;
+        }
     }
 }

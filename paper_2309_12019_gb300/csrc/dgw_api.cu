@@ -9,6 +9,7 @@
 #include <set>
 #include <string>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 #include <algorithm>
 #include <vector>
@@ -1734,20 +1735,30 @@ extern "C" dgw_status dgw_adjoint_step_stages(dgw_ctx* c, const void* U_n, const
     return DGW_OK;
 }
 
-template <typename Real>
-__global__ void misfit_kernel(const Real* U, const Real* Ut, Real* grad, int64_t E, int K, int n1, int dim,
-                              double h, double* partial)
+// Mass of every mode of a cell, int phi_k^2 (a table: its divisions, done per coefficient, held the
+// FP64 pipe for most of the kernel's 128 us on 512^2 Q2 cells)
+struct MassTable {
+    double m[4 * kMaxK];
+};
+
+template <typename Real, int K>
+__global__ void misfit_kernel(const Real* U, const Real* Ut, Real* grad, int64_t E,
+                              const __grid_constant__ MassTable t, double* partial)
 {
     __shared__ double sh[kMassThreads];
     double s = 0.0;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x) {
+        Real u[K], ut[K];
+#pragma unroll
         for (int k = 0; k < K; ++k) {
-            const int i = k % n1, j = k / n1;
-            double m = 0.5 * h * 2.0 / (2 * i + 1);            // mass of P_i on a cell of width h
-            if (dim == 2) m *= 0.5 * h * 2.0 / (2 * j + 1);
-            const double d = (double)U[k * E + e] - (double)Ut[k * E + e];
-            s += 0.5 * m * d * d;
-            if (grad) grad[k * E + e] = (Real)(m * d);
+            u[k] = U[k * E + e];
+            ut[k] = Ut[k * E + e];
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const double d = (double)u[k] - (double)ut[k], md = t.m[k] * d;
+            s = fma(0.5 * md, d, s);
+            if (grad) grad[k * E + e] = (Real)md;
         }
     }
     sh[threadIdx.x] = s;
@@ -1766,14 +1777,32 @@ extern "C" dgw_status dgw_misfit(dgw_ctx* c, const void* U, const void* U_target
     if (st != DGW_OK) return st;
     if (!U || !U_target || !host_J) return fail(DGW_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    if (c->params.prec == DGW_FP64)
-        misfit_kernel<double><<<kMassBlocks, kMassThreads, 0, s>>>((const double*)U, (const double*)U_target,
-                                                                   (double*)grad, c->E, c->K, c->p + 1, c->mesh.dim,
-                                                                   c->h, c->partial);
-    else
-        misfit_kernel<float><<<kMassBlocks, kMassThreads, 0, s>>>((const float*)U, (const float*)U_target,
-                                                                 (float*)grad, c->E, c->K, c->p + 1, c->mesh.dim,
-                                                                 c->h, c->partial);
+    MassTable t;
+    const int n1 = c->p + 1;
+    for (int k = 0; k < c->K; ++k) {
+        t.m[k] = 0.5 * c->h * 2.0 / (2 * (k % n1) + 1);                             // mass of P_i on a cell of width h
+        if (c->mesh.dim == 2) t.m[k] *= 0.5 * c->h * 2.0 / (2 * (k / n1) + 1);
+    }
+    auto run = [&](auto kc) {
+        constexpr int kK = decltype(kc)::value;
+        if (c->params.prec == DGW_FP64)
+            misfit_kernel<double, kK><<<kMassBlocks, kMassThreads, 0, s>>>((const double*)U, (const double*)U_target,
+                                                                           (double*)grad, c->E, t, c->partial);
+        else
+            misfit_kernel<float, kK><<<kMassBlocks, kMassThreads, 0, s>>>((const float*)U, (const float*)U_target,
+                                                                          (float*)grad, c->E, t, c->partial);
+    };
+    switch (c->K) {            // (p + 1)^dim times the components
+    case 2: run(std::integral_constant<int, 2>()); break;
+    case 3: run(std::integral_constant<int, 3>()); break;
+    case 4: run(std::integral_constant<int, 4>()); break;
+    case 6: run(std::integral_constant<int, 6>()); break;
+    case 9: run(std::integral_constant<int, 9>()); break;
+    case 12: run(std::integral_constant<int, 12>()); break;
+    case 16: run(std::integral_constant<int, 16>()); break;
+    case 36: run(std::integral_constant<int, 36>()); break;
+    default: run(std::integral_constant<int, 64>()); break;
+    }
     DGW_CUDA(cudaGetLastError());
     mass_final_kernel<<<1, kMassThreads, 0, s>>>(c->partial, kMassBlocks, 1.0, c->mass_dev);
     DGW_CUDA(cudaGetLastError());
