@@ -6,7 +6,7 @@
 // k = i + (p+1) j of component comp of cell e at row comp K + k, K = (p+1)^2.
 // One CTA of 32 x EY threads owns a tile of as many cells, one per thread:
 //   0. the tile's coefficients and a one-cell face halo (all four components) are
-//      staged in shared memory by coalesced row loads; halo cells beyond a periodic side
+//      staged in shared memory by asynchronous copies of words; halo cells beyond a periodic side
 //      are its images, beyond a wall or an outflow side they are absent; in float the
 //      Un coefficients of the tile start to arrive by cp.async
 //   1. per cell: the sensor of Sec. 4 on the density, the volume term at the (p+2)^2
@@ -25,7 +25,9 @@
 // with the tile's Un in shared memory 3 CTAs of 4 rows fitted (12 warps, issue active 59 %); Un
 // is now prefetched into L2 and read into registers after the faces, which makes room for 16
 // warps, and the taller tile has fewer halo cells and faces per cell.  Kelvin-Helmholtz 2048^2, p = 2,
-// FP32: 746 -> 680 us a stage; triple point 896 x 384: 69 -> 66 us.
+// FP32: 746 -> 680 us a stage; triple point 896 x 384: 69 -> 66 us.  The tile's coefficients arrive by
+// cp.async, all in flight at once; loads into registers stalled the warps for a third of the time
+// (675 -> 629 us and 62.7 -> 56.7 us).
 using R2 = std::conditional_t<kF32, float2, double2>;   // a pair of state components
 constexpr int EX = kTileX2, EHX = EX + 2;               // tile columns, staged columns
 template <int P> constexpr int euler2_rows() { return kF32 && P <= 2 ? 8 : kTileY2; }
@@ -166,26 +168,27 @@ __global__ void __launch_bounds__(EX * euler2_rows<P>(), euler2_blocks<P>()) eul
     const int tid = threadIdx.x;
     const int64_t E = A.E;
     const int tx0 = blockIdx.x * EX, ty0 = blockIdx.y * EY;
-    // ---- 0. stage the tile and its face halo ----
+    // ---- 0. stage the tile and its face halo: asynchronous copies, all in flight at once ----
     for (int idx = tid; idx < EHY * EHX; idx += ENT) {
         const int r = idx / EHX, cc = idx - r * EHX;
         const bool corner = (r == 0 || r == EHY - 1) && (cc == 0 || cc == EHX - 1);
         const int gx = wrap_x(A, tx0 - 1 + cc), gy = wrap_y(A, ty0 - 1 + r);
         const bool ok = !corner && gx >= 0 && gy >= 0;
         S.has[r][cc] = ok;
-        const Real* src = A.Uk + (ok ? (int64_t)gy * A.nx + gx : 0);
+        if (ok) {
+            const Real* src = A.Uk + (int64_t)gy * A.nx + gx;
 #pragma unroll
-        for (int pr = 0; pr < 2; ++pr)
+            for (int comp = 0; comp < 4; ++comp)
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                R2 v = vbc<R2>(0);
-                if (ok) {
-                    v.x = src[(int64_t)(2 * pr * K + k) * E];
-                    v.y = src[(int64_t)((2 * pr + 1) * K + k) * E];
-                }
-                S.u[pr][k][r][cc] = v;
-            }
+                for (int k = 0; k < K; ++k) cp_async_word(&lane(S.u[comp >> 1][k][r][cc], comp & 1), src + (int64_t)(comp * K + k) * E);
+        } else {
+#pragma unroll
+            for (int pr = 0; pr < 2; ++pr)
+#pragma unroll
+                for (int k = 0; k < K; ++k) S.u[pr][k][r][cc] = vbc<R2>(0);
+        }
     }
+    cp_async_commit();
     const int lx = tid % EX, ly = tid / EX;
     const int gx = tx0 + lx, gy = ty0 + ly;
     const bool in = gx < A.nx && gy < A.ny;
@@ -201,6 +204,7 @@ __global__ void __launch_bounds__(EX * euler2_rows<P>(), euler2_blocks<P>()) eul
             if (((uintptr_t)a & 127u) != 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(a + last));
         }
     }
+    cp_async_wait_all();
     __syncthreads();
 
     // ---- 1. sensor of the density; volume term; lambda_e over the volume points ----
