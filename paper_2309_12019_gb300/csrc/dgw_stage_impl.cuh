@@ -1456,8 +1456,20 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
         if (in[l] && lane(chk, l) != lane(chk, l)) atomicOr(A.flag, 1u);
 }
 
-template <int P, int FLUX, int MODE>
-__global__ void __launch_bounds__(NTS, LS == 2 ? 512 / NTS : (kF32 ? 6 : 384 / NTS)) stage_kernel(const __grid_constant__ KParams A)
+// Resident CTAs per SM that the registers are sized for.  Float 2D: two (128 registers, no spills)
+// or, with `dense`, three at p = 2 (80, up to 24 bytes of spills) and four at p = 1 (64), for launches
+// of more CTAs than that would leave in one round.  p = 2 FP32, us a stage, two / three CTAs: KPP 256^2
+// 10.2 / 12.4, 512^2 19.3 / 17.5, 1024^2 59.2 / 50.4; Burgers 512^2 25.5 / 25.9, 1024^2 68.2 / 60.2.
+// p = 1, three / four CTAs: Burgers 333 x 217 9.4 / 11.0, 1024^2 34.0 / 31.3.
+template <int P>
+constexpr int stage_blocks(bool dense)
+{
+    if (LS == 2) return P == 3 ? 2 : (P == 2 ? (dense ? 3 : 2) : (dense ? 4 : 3));
+    return kF32 ? 6 : 3;
+}
+
+template <int P, int FLUX, int MODE, bool DENSE>
+__global__ void __launch_bounds__(NTS, stage_blocks<P>(DENSE)) stage_kernel(const __grid_constant__ KParams A)
 {
     pdl_begin();
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1996,11 +2008,14 @@ static int sm_count()
     return nsm[dev];
 }
 
-// The persistent kernel pays where every SM walks several of its tiles; on smaller meshes
-// (fewer than four tiles of 32 x 32 cells per SM) the tile kernel's smaller tiles keep
-// more SMs busy.
+// The persistent kernel pays for rotation at p = 3 where every SM walks several of its tiles (1024^2:
+// 74.9 us a stage against the tile kernel's 76.6, 2048^2: 267 against 288).  Elsewhere the tile kernel
+// is as fast or faster: KPP p = 3 1024^2 96.8 against 97.5, Burgers p = 3 111 against 131, advection p = 3
+// 86.9 against 109, and at p <= 2 it has more warps per SM (1024^2 p = 2 KPP 50 against 61).
+template <int P, int FLUX>
 static bool persistent_pays(int nx, int ny)
 {
+    if (P < 3 || FLUX != FLUX_ROTATION) return false;
     const int nsm = sm_count();
     const long long ntiles = (long long)((nx + TX - 1) / TX) * ((ny + kPRows - 1) / kPRows);
     return nsm > 0 && ntiles >= 4LL * nsm;
@@ -2025,6 +2040,25 @@ static cudaError_t launch_persistent(const KParams& a, bool pdl, cudaStream_t st
 }
 #endif
 
+template <int P, int FLUX, int MODE, bool DENSE>
+static cudaError_t launch_tile(const KParams& a, dim3 grid, size_t smem, bool pdl, cudaStream_t st)
+{
+    // once per instantiation and device: opt in to more than 48 KB of dynamic shared
+    // memory where needed, and prefer the largest shared-memory carveout (several tiles per SM)
+    static bool opted[64] = {false};
+    const int dev = cur_device();
+    if (!opted[dev]) {
+        const void* fn = (const void*)stage_kernel<P, FLUX, MODE, DENSE>;
+        cudaError_t e = cudaSuccess;
+        if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        opted[dev] = true;
+    }
+    return launch_k(stage_kernel<P, FLUX, MODE, DENSE>, grid, NTS, smem, pdl, st, a);
+}
+
 template <int P, int FLUX>
 static cudaError_t launch_pf(const StageArgs& s, int mode, cudaStream_t st)
 {
@@ -2036,27 +2070,19 @@ static cudaError_t launch_pf(const StageArgs& s, int mode, cudaStream_t st)
     dim3 grid((s.nx + TX - 1) / TX, grows);
     if (grid.x == 0 || grid.y == 0) return cudaSuccess;
     const size_t smem = sizeof(TileSmem<P, LS, TYS>);
-    // once per instantiation and device: opt in to more than 48 KB of dynamic shared
-    // memory where needed, and prefer the largest shared-memory carveout (several tiles per SM)
-    static bool opted[64][2] = {{false, false}};
-    const int dev = cur_device();
-    if (!opted[dev][mode]) {
-        const void* fn = mode == 0 ? (const void*)stage_kernel<P, FLUX, 0> : (const void*)stage_kernel<P, FLUX, 1>;
-        cudaError_t e = cudaSuccess;
-        if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        opted[dev][mode] = true;
-    }
 #if DGW_DIM == 2
     if constexpr (kF32) {
         if (mode == 0 && s.tmap_p && s.tile_row0 == 0 && s.tile_rows == 0 && (!a.has_un || a.use_p_un) &&
-            (s.kernel_choice == 2 || persistent_pays(s.nx, s.ny)))
+            (s.kernel_choice == 2 || persistent_pays<P, FLUX>(s.nx, s.ny)))
             return launch_persistent<P, FLUX>(a, s.pdl != 0, st);
     }
+    if constexpr (stage_blocks<P>(true) != stage_blocks<P>(false)) {
+        if (mode == 0 && (long long)grid.x * grid.y > (long long)stage_blocks<P>(false) * sm_count())
+            return launch_tile<P, FLUX, 0, true>(a, grid, smem, s.pdl != 0, st);
+    }
 #endif
-    return launch_k(mode == 0 ? stage_kernel<P, FLUX, 0> : stage_kernel<P, FLUX, 1>, grid, NTS, smem, s.pdl != 0, st, a);
+    return mode == 0 ? launch_tile<P, FLUX, 0, false>(a, grid, smem, s.pdl != 0, st)
+                     : launch_tile<P, FLUX, 1, false>(a, grid, smem, s.pdl != 0, st);
 }
 
 template <int P>
