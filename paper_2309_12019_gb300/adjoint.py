@@ -5,7 +5,9 @@ rollout(ctx, U0, dt, nsteps, every) advances U0 by nsteps SSP-RK3 steps and keep
 checkpoint every `every` steps; its backward pass recomputes each segment from its
 checkpoint, keeping every step's state and its two stage states (dgw_rk_step_stages),
 and runs dgw_adjoint_step_stages through the segment in reverse, so that no stage is
-evaluated twice in the backward pass.
+evaluated twice in the backward pass.  The last segment, with which the backward pass
+begins, is kept by the forward pass when a gradient is asked for: its states are not
+recomputed, and the largest memory in use (the checkpoints and one segment) is the same.
 misfit(ctx, U, U_target) is J = 1/2 int (U_h - U_target)^2 with dJ/dU from dgw_misfit.
 All arithmetic runs in the library's kernels; this module only orders the calls.
 """
@@ -14,41 +16,51 @@ from __future__ import annotations
 import torch
 
 
+def _segment(dctx, U, dt, n, last_state):
+    """n steps from U keeping every step's (U_n, U_1, U_2); and the state after them, None
+    unless last_state (the last step's third stage is then skipped)."""
+    steps = []
+    for i in range(n):
+        U1, U2 = torch.empty_like(U), torch.empty_like(U)
+        nxt = torch.empty_like(U) if last_state or i < n - 1 else None
+        dctx.rk_step_stages(U, dt, U1, U2, nxt)
+        steps.append((U, U1, U2))
+        U = nxt
+    return steps, U
+
+
 class _Rollout(torch.autograd.Function):
     @staticmethod
     def forward(ctx_, U0, dctx, dt, nsteps, every):
         U = U0.detach().clone().contiguous()
-        checkpoints = [U.clone()]
-        done = 0
+        # (what has no adjoint has no stage states either: its forward pass takes plain steps)
+        keep = ctx_.needs_input_grad[0] and dctx.problem.rk_order == 3 and "state" not in dctx.problem.bc
+        checkpoints, last, done = [], None, 0
         while done < nsteps:
             n = min(every, nsteps - done)
-            dctx.rk_step(U, dt, n)
             done += n
-            if done < nsteps:
+            if keep and done == nsteps:
+                last, U = _segment(dctx, U, dt, n, True)
+            else:
                 checkpoints.append(U.clone())
+                dctx.rk_step(U, dt, n)
         ctx_.dctx, ctx_.dt, ctx_.nsteps, ctx_.every = dctx, dt, nsteps, every
-        ctx_.checkpoints = checkpoints
+        ctx_.checkpoints, ctx_.last = checkpoints, last
         return U
 
     @staticmethod
     def backward(ctx_, gout):
         dctx, dt, nsteps, every = ctx_.dctx, ctx_.dt, ctx_.nsteps, ctx_.every
         lam = gout.detach().clone().contiguous()
-        for seg in reversed(range(len(ctx_.checkpoints))):
-            start = seg * every
-            n = min(every, nsteps - start)
-            states = [ctx_.checkpoints[seg]]
-            stages = []
-            for i in range(n):
-                U1, U2 = torch.empty_like(lam), torch.empty_like(lam)
-                nxt = torch.empty_like(lam) if i < n - 1 else None   # the last step needs no U^{n+1}
-                dctx.rk_step_stages(states[-1], dt, U1, U2, nxt)
-                stages.append((U1, U2))
-                if nxt is not None:
-                    states.append(nxt)
-            for Un, (U1, U2) in zip(reversed(states), reversed(stages)):
+        steps, ctx_.last = ctx_.last, None
+        segments = list(range(len(ctx_.checkpoints)))
+        while steps or segments:
+            if not steps:
+                seg = segments.pop()
+                steps, _ = _segment(dctx, ctx_.checkpoints[seg], dt, min(every, nsteps - seg * every), False)
+            while steps:
+                Un, U1, U2 = steps.pop()
                 dctx.adjoint_step_stages(Un, U1, U2, lam, lam, dt)
-            del states, stages
         ctx_.checkpoints = None
         return lam, None, None, None, None
 
