@@ -237,12 +237,12 @@ dgw_status dgw_sync_status(dgw_ctx* ctx, void* stream);
 dgw_status dgw_debug(dgw_ctx* ctx, int wait_limit);
 
 /* Which kernel runs the context's whole-mesh stage launches on 2D FP32 meshes whose rows
- * are 16-byte multiples: 0 (the default) the persistent kernel (one 512-thread CTA per
- * SM walking tiles of 32 x 32 cells, the next tile's data loaded during the current
- * one's arithmetic) when the mesh has at least four such tiles per SM, else the tile
- * kernel (one CTA per 32 x 16-cell tile); 1 always the tile kernel; 2 the persistent
- * kernel wherever it applies.  The two kernels give bitwise the same results.  Any
- * other choice is DGW_EINVAL.  Drops the context's cached graphs. */
+ * are 16-byte multiples: 0 (the default) the faster one as measured: the persistent kernel
+ * (one 512-thread CTA per SM walking tiles of 32 x 32 cells, the next tile's data loaded
+ * during the current one's arithmetic) for the rotation flux at p = 3 on meshes of at least
+ * four such tiles per SM, else the tile kernel (one CTA per 32 x 16-cell tile); 1 always the
+ * tile kernel; 2 the persistent kernel wherever it applies.  The two kernels give bitwise the
+ * same results.  Any other choice is DGW_EINVAL.  Drops the context's cached graphs. */
 dgw_status dgw_set_stage_kernel(dgw_ctx* ctx, int choice);
 
 /* ------------------------------------------------------------------------------------
@@ -332,7 +332,7 @@ dgw_status dgw_batch_autotune(dgw_batch* b, void* U, int steps, int* chosen_chun
 /* Schedule of the group of instances of dimension dim and degree p: the tile height of its
  * kernel (*rows) and the tiles per work item (*chunk).  Either pointer may be NULL.  Until
  * an autotune or dgw_batch_set_schedule: 1D items of 2 tiles; 2D float tiles of 8 rows and
- * items of 16 tiles; 2D double tiles of 4 rows and items of 16 tiles. */
+ * items of 16 tiles (p = 1: 8); 2D double tiles of 4 rows and items of 16 tiles. */
 dgw_status dgw_batch_schedule(const dgw_batch* b, int dim, int p, int* rows, int* chunk);
 
 /* Sets that schedule (a tile height that is built, chunk >= 1; DGW_EINVAL otherwise), e.g.
