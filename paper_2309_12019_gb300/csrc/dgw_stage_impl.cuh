@@ -125,6 +125,7 @@ struct KParams {
     int cg_loads;        // load Uk / Un through L2 only (data written earlier in the same launch)
     int wait_limit;      // polls of a TMA mbarrier wait before it gives up (kWaitLimit)
     int tile_row0;       // first tile row of a stage launch over a band of rows
+    int round_tiles;     // 2D Euler kernel: tiles that run at once (0: no prefetch of the next ones)
     const Real* Uk;
     const Real* Un;
     Real* Uout;
@@ -1608,6 +1609,17 @@ static int cur_device()
     return dev;
 }
 
+// SMs of the current device (0 if it cannot be read)
+[[maybe_unused]] static int sm_count()
+{
+    static int nsm[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (nsm[dev] == 0 && cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        nsm[dev] = 0;
+    return nsm[dev];
+}
+
 static KParams make_params(const StageArgs& s)
 {
     KParams a;
@@ -1997,17 +2009,6 @@ __device__ __forceinline__ double max_nan(double a, double b)
 #endif
 
 #if DGW_DIM == 2
-// SMs of the current device (0 if it cannot be read)
-static int sm_count()
-{
-    static int nsm[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    if (nsm[dev] == 0 && cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        nsm[dev] = 0;
-    return nsm[dev];
-}
-
 // The persistent kernel pays for rotation at p = 3 where every SM walks several of its tiles (1024^2:
 // 74.9 us a stage against the tile kernel's 76.6, 2048^2: 267 against 288).  Elsewhere the tile kernel
 // is as fast or faster: KPP p = 3 1024^2 96.8 against 97.5, Burgers p = 3 111 against 131, advection p = 3
