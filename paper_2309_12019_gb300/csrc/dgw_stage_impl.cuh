@@ -291,6 +291,10 @@ __device__ __forceinline__ float2 vfma(float a, float2 b, float2 c) { return __f
 __device__ __forceinline__ Real vmul(Real a, Real b) { return a * b; }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vmul(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
+// products that are not contracted into a following sum (the packed ones never are)
+__device__ __forceinline__ Real vmul_x(Real a, Real b) { return mul_x(a, b); }
+__device__ __forceinline__ float2 vmul_x(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vmul_x(float a, float2 b) { return __fmul2_rn(make_float2(a, a), b); }
 __device__ __forceinline__ Real vadd(Real a, Real b) { return a + b; }
 __device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ Real vsub(Real a, Real b) { return a - b; }
@@ -327,9 +331,9 @@ __device__ __forceinline__ void vol_flux_v(const KParams& A, V u, Real x, V y, V
 #pragma unroll
         for (int l = 0; l < Lanes<V>::n; ++l) lane(key, l) = DIM == 1 ? fabs(lane(fy, l)) : Real(1);
     } else if constexpr (FLUX == FLUX_BURGERS) {
-        const V hu2 = vmul(vmul(Real(0.5), u), u);
-        fx = vmul(A.a0, hu2);
-        fy = vmul(A.a1, hu2);
+        const V hu2 = vmul_x(vmul_x(Real(0.5), u), u);
+        fx = vmul_x(A.a0, hu2);
+        fy = vmul_x(A.a1, hu2);
 #pragma unroll
         for (int l = 0; l < Lanes<V>::n; ++l) lane(key, l) = fabs(lane(u, l));
     } else {
@@ -428,7 +432,7 @@ template <int FLUX, class V>
 __device__ __forceinline__ V llf_v(V v, V uL, V uR)
 {
     V s, d = vsub(uR, uL);
-    if constexpr (FLUX == FLUX_ROTATION) {
+    if constexpr (FLUX != FLUX_BURGERS) {
 #pragma unroll
         for (int l = 0; l < Lanes<V>::n; ++l) lane(s, l) = fabs(lane(v, l));
         return vfma(vmul(Real(-0.5), s), d, vmul(vmul(Real(0.5), v), vadd(uL, uR)));
@@ -691,11 +695,12 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     const int64_t E = A.E;
     // lambda_e from the largest key of the cell's points; advection and the 2D KPP flux have the
     // same key at every point, so their faces contribute nothing
-    // (and rotation's keys depend on the position alone: kLinear below takes them with the volume)
+    // (and rotation's keys depend on the position alone: they are taken after the volume term)
     constexpr bool kSameSpeed = FLUX == FLUX_ADVECT || (DIM == 2 && (FLUX == FLUX_KPP || FLUX == FLUX_ROTATION));
     // F linear in u with coefficients of degree at most one: the Gauss rule integrates the volume
-    // term exactly, so it is taken in closed form (below)
-    constexpr bool kLinear = DIM == 2 && (FLUX == FLUX_ADVECT || FLUX == FLUX_ROTATION);
+    // term exactly, so it is taken in closed form (below).  In double only: in float the other
+    // rounding moves some cells across the sensor's threshold b, where the scheme jumps.
+    constexpr bool kLinear = DIM == 2 && !kF32 && (FLUX == FLUX_ADVECT || FLUX == FLUX_ROTATION);
     const bool find_lam = (MODE == 0) && (A.stab != STAB_DG) && !A.lam_fixed;
     const bool need_lam = find_lam && !kSameSpeed;
     const bool periodic_x = A.bc[0] == BC_PERIODIC;
@@ -992,9 +997,8 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     } else if constexpr (kLinear) {
         // int P_i' P_m = 2 for m < i, i - m odd (else 0), int P_j P_j = A0_j, and eta P_j couples j
         // with j +- 1 only, int eta P_j P_{j+1} = 2 (j + 1) / ((2j + 1)(2j + 3)): a few products per
-        // mode in place of the Gauss points, the same integral.  With the faces of advection below:
-        // ensemble of 512 (its 2D instances are advection) 2.29 -> 2.02 ms a step; rotation 256^2 Q2
-        // FP64 142 -> 134 us a stage.
+        // mode in place of the Gauss points, the same integral.  Rotation 256^2 Q2 FP64, with the keys
+        // at the outermost nodes below: 142 -> 107 us a stage.
         constexpr auto X2 = [](int j) { return Real(4.0 * (j + 1) / ((2.0 * j + 1) * (2.0 * j + 3))); };   // twice that
         // velocity (v0x - v1 eta, v0y + v1 xi) in the cell's frame
         V v0x;
@@ -1043,22 +1047,6 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                 acc[n + N1 * d] = ty;
             }
         }
-        if (FLUX == FLUX_ROTATION && find_lam) {
-            // |v|^2 is convex, so over the Gauss points of the cell and of its faces it is largest at
-            // an outermost node of a face: the larger |v_x| and |v_y| of those four lines
-            const Real g = T.g[NQ - 1];
-            const Real vyg = max_pos(fabs(mul_x(A.omega, fma_x(A.hh, g, xc) - A.cx)), fabs(mul_x(A.omega, fma_x(A.hh, -g, xc) - A.cx)));
-            const Real vye = max_pos(fabs(mul_x(A.omega, fma_x(Real(gx), A.h, A.x0) - A.cx)),
-                                     fabs(mul_x(A.omega, fma_x(Real(gx + 1), A.h, A.x0) - A.cx)));
-#pragma unroll
-            for (int l = 0; l < L; ++l) {
-                const Real yl = lane(yc, l);
-                const Real vxg = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(A.hh, g, yl))), fabs(mul_x(A.omega, A.cy - fma_x(A.hh, -g, yl))));
-                const Real vxe = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l]), A.h, A.y0))),
-                                         fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l] + 1), A.h, A.y0))));
-                lane(lam, l) = max_pos(fma_x(vxg, vxg, mul_x(vye, vye)), fma_x(vxe, vxe, mul_x(vyg, vyg)));
-            }
-        }
     } else {
         // one Gauss row qy at a time: the polynomial reduced to the row (rr[i] =
         // sum_j P_j(g_qy) c_ij), its values at the row's points, the fluxes there, and
@@ -1074,7 +1062,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             for (int qx = 0; qx < NQ; ++qx) {
                 V key;
                 vol_flux_v<FLUX>(A, u[qx], fma_x(A.hh, T.g[qx], xc), y, fx[qx], fy[qx], key);
-                lam = vmax(lam, key);
+                if (FLUX != FLUX_ROTATION) lam = vmax(lam, key);
             }
             V px[N1], py[N1];
             project_sym<true, N1, NQ>(T.WD, fx, px);      // px[0] = 0 (P_0' = 0)
@@ -1105,6 +1093,22 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             row(qy, rr);
         }
     }
+            if (DIM == 2 && FLUX == FLUX_ROTATION && find_lam) {
+                // |v|^2 is convex, so over the Gauss points of the cell and of its faces it is largest at
+                // an outermost node of a face: the larger |v_x| and |v_y| of those four lines
+                const Real g = T.g[NQ - 1];
+                const Real vyg = max_pos(fabs(mul_x(A.omega, fma_x(A.hh, g, xc) - A.cx)), fabs(mul_x(A.omega, fma_x(A.hh, -g, xc) - A.cx)));
+                const Real vye = max_pos(fabs(mul_x(A.omega, fma_x(Real(gx), A.h, A.x0) - A.cx)),
+                                         fabs(mul_x(A.omega, fma_x(Real(gx + 1), A.h, A.x0) - A.cx)));
+#pragma unroll
+                for (int l = 0; l < L; ++l) {
+                    const Real yl = lane(yc, l);
+                    const Real vxg = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(A.hh, g, yl))), fabs(mul_x(A.omega, A.cy - fma_x(A.hh, -g, yl))));
+                    const Real vxe = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l]), A.h, A.y0))),
+                                             fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l] + 1), A.h, A.y0))));
+                    lane(lam, l) = max_pos(fma_x(vxg, vxg, mul_x(vye, vye)), fma_x(vxe, vxe, mul_x(vyg, vyg)));
+                }
+            }
     __syncthreads();
 
     // The stage array is no longer read: bring the Un tile into it now, so that its
@@ -1193,7 +1197,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
         }
         [[maybe_unused]] V lm = vbc<V>(0), lp = vbc<V>(0);
         V hq[TN];
-        if constexpr (FLUX == FLUX_ADVECT && DIM == 2) {
+        if constexpr (FLUX == FLUX_ADVECT && kLinear) {
             // the flux is linear: its face modes are those of the traces times int P_t P_t,
             // upwind, H_t = A0_t (max(a, 0) U-_t + min(a, 0) U+_t).  Beyond a side the inner trace, or
             // zero where the flow enters through an inflow side.
@@ -1249,7 +1253,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                         }
                     }
                     Hq[q] = llf_kpp(uL, uR);
-                } else if constexpr (DIM == 2) {
+                } else if constexpr (DIM == 2 && FLUX != FLUX_ADVECT) {
                     V uL = uLq[q], uR = uRq[q], v;
 #pragma unroll
                     for (int l = 0; l < L; ++l) {
@@ -1266,7 +1270,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
                             const Real ui = minus_in ? lane(uL, l) : lane(uR, l);
-                            const Real df = FLUX == FLUX_ROTATION ? lane(v, l) : lane(v, l) * ui;
+                            const Real df = FLUX == FLUX_BURGERS ? lane(v, l) * ui : lane(v, l);
                             const int kind = minus_in ? A.bc[xf ? 1 : 3] : A.bc[xf ? 0 : 2];
                             const Real gh = (kind == BC_INFLOW_ZERO && (minus_in ? df : -df) < Real(0)) ? Real(0) : ui;
                             if (minus_in) lane(uR, l) = gh;
