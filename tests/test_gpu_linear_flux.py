@@ -1,4 +1,4 @@
-"""The closed-form volume and face terms of the linear fluxes (2D advection, rotation) against the
+"""The closed-form volume and face terms of the linear fluxes (2D, double) against the
 oracle's quadrature: velocities of either sign and zero along an axis, every kind of side, rotation
 centres inside and far outside the mesh, ragged tiles."""
 import numpy as np
