@@ -747,6 +747,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
             if (w.in) v[r] = fma(cn, un[r], fma(cl, mk[r] * x, ck * v[r]));
             bad = bad || not_finite(v[r]);
         }
+        __syncwarp();          // the next stage's modes replace those that other lanes read above
         buf ^= 1;
     });
     if (!w.in) return;
