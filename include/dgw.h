@@ -280,7 +280,8 @@ dgw_status dgw_rk_step_stages(dgw_ctx* ctx, const void* U, double dt, void* U1, 
 dgw_status dgw_adjoint_step_stages(dgw_ctx* ctx, const void* U_n, const void* U1, const void* U2,
                                    const void* lam_np1, void* lam_n, double dt, void* stream);
 
-/* Misfit J = 1/2 int (U_h - U_target,h)^2 dx (exact: mass-matrix weighted) in double,
+/* Misfit J = 1/2 int (U_h - U_target,h)^2 dx (exact: mass-matrix weighted; the Euler system:
+ * summed over the conserved variables) in double,
  * and optionally grad = dJ/dU = M (U - U_target) (device, K*E, may be NULL).  Blocks
  * until *host_J is set. */
 dgw_status dgw_misfit(dgw_ctx* ctx, const void* U, const void* U_target, double* host_J, void* grad,

@@ -1785,7 +1785,7 @@ extern "C" dgw_status dgw_misfit(dgw_ctx* c, const void* U, const void* U_target
     const int n1 = c->p + 1;
     for (int k = 0; k < c->K; ++k) {
         t.m[k] = 0.5 * c->h * 2.0 / (2 * (k % n1) + 1);                             // mass of P_i on a cell of width h
-        if (c->mesh.dim == 2) t.m[k] *= 0.5 * c->h * 2.0 / (2 * (k / n1) + 1);
+        if (c->mesh.dim == 2) t.m[k] *= 0.5 * c->h * 2.0 / (2 * (k / n1 % n1) + 1);  // n1 n1 rows a component
     }
     auto run = [&](auto kc) {
         constexpr int kK = decltype(kc)::value;
