@@ -31,10 +31,10 @@ def _segment(dctx, U, dt, n, last_state):
 
 class _Rollout(torch.autograd.Function):
     @staticmethod
-    def forward(ctx_, U0, dctx, dt, nsteps, every):
+    def forward(ctx_, U0, dctx, dt, nsteps, every, grad):
         U = U0.detach().clone().contiguous()
         # (what has no adjoint has no stage states either: its forward pass takes plain steps)
-        keep = ctx_.needs_input_grad[0] and dctx.problem.rk_order == 3 and "state" not in dctx.problem.bc
+        keep = grad and dctx.problem.rk_order == 3 and "state" not in dctx.problem.bc
         checkpoints, last, done = [], None, 0
         while done < nsteps:
             n = min(every, nsteps - done)
@@ -62,7 +62,7 @@ class _Rollout(torch.autograd.Function):
                 Un, U1, U2 = steps.pop()
                 dctx.adjoint_step_stages(Un, U1, U2, lam, lam, dt)
         ctx_.checkpoints = None
-        return lam, None, None, None, None
+        return lam, None, None, None, None, None
 
 
 class _Misfit(torch.autograd.Function):
@@ -80,7 +80,9 @@ class _Misfit(torch.autograd.Function):
 
 
 def rollout(dctx, U0, dt: float, nsteps: int, every: int = 20):
-    return _Rollout.apply(U0, dctx, float(dt), int(nsteps), int(every))
+    # (inside forward() gradients are off, and needs_input_grad ignores no_grad)
+    grad = U0.requires_grad and torch.is_grad_enabled()
+    return _Rollout.apply(U0, dctx, float(dt), int(nsteps), int(every), grad)
 
 
 def misfit(dctx, U, U_target):

@@ -46,3 +46,12 @@ def test_rollout_without_an_adjoint_steps_forward(kw):
     with torch.no_grad():
         U = adjoint.rollout(c, torch.ones(2, dtype=torch.float64, requires_grad=True), 0.1, 5, 2)
     assert float(U[0]) == 1.5 ** 5
+
+
+def test_rollout_without_a_gradient_keeps_no_stages():
+    U0 = torch.ones(2, dtype=torch.float64, requires_grad=True)
+    c = Ctx()
+    with torch.no_grad():
+        assert float(adjoint.rollout(c, U0, 0.1, 5, 2)[0]) == 1.5 ** 5
+    adjoint.rollout(c, U0.detach(), 0.1, 5, 2)
+    assert c.kept == 0
