@@ -6,14 +6,38 @@ checkpoint every `every` steps; its backward pass recomputes each segment from i
 checkpoint, keeping every step's state and its two stage states (dgw_rk_step_stages),
 and runs dgw_adjoint_step_stages through the segment in reverse, so that no stage is
 evaluated twice in the backward pass.  The last segment, with which the backward pass
-begins, is kept by the forward pass when a gradient is asked for: its states are not
-recomputed, and the largest memory in use (the checkpoints and one segment) is the same.
+begins, is kept by the forward pass when a gradient is asked for, so that its states are
+not recomputed.  A context holds one such segment at most, that of its latest rollout: an
+earlier one, of a graph that was chained or is still waiting for its backward pass, falls
+back to its checkpoint.  So the largest memory in use, the checkpoints and one segment, is
+that of a backward pass which recomputes every segment; it is held from the forward pass on.
 misfit(ctx, U, U_target) is J = 1/2 int (U_h - U_target)^2 with dJ/dU from dgw_misfit.
 All arithmetic runs in the library's kernels; this module only orders the calls.
 """
 from __future__ import annotations
 
+import weakref
+
 import torch
+
+
+class _Kept:
+    """The stages of a rollout's last segment, until its backward pass takes them or the next
+    rollout on the context drops them."""
+
+    def __init__(self, dctx, steps):
+        self.steps = steps
+        dctx.kept_segment = weakref.ref(self)
+
+    def take(self):
+        steps, self.steps = self.steps, None
+        return steps
+
+    @staticmethod
+    def drop(dctx):
+        kept = getattr(dctx, "kept_segment", lambda: None)()
+        if kept is not None:
+            kept.take()
 
 
 def _segment(dctx, U, dt, n, last_state):
@@ -40,7 +64,10 @@ class _Rollout(torch.autograd.Function):
             n = min(every, nsteps - done)
             done += n
             if keep and done == nsteps:
-                last, U = _segment(dctx, U, dt, n, True)
+                _Kept.drop(dctx)
+                checkpoints.append(U)
+                steps, U = _segment(dctx, U, dt, n, True)
+                last = _Kept(dctx, steps)
             else:
                 checkpoints.append(U.clone())
                 dctx.rk_step(U, dt, n)
@@ -52,11 +79,10 @@ class _Rollout(torch.autograd.Function):
     def backward(ctx_, gout):
         dctx, dt, nsteps, every = ctx_.dctx, ctx_.dt, ctx_.nsteps, ctx_.every
         lam = gout.detach().clone().contiguous()
-        steps, ctx_.last = ctx_.last, None
-        segments = list(range(len(ctx_.checkpoints)))
-        while steps or segments:
-            if not steps:
-                seg = segments.pop()
+        for seg in reversed(range(len(ctx_.checkpoints))):
+            steps = ctx_.last.take() if ctx_.last is not None else None
+            ctx_.last = None
+            if steps is None:
                 steps, _ = _segment(dctx, ctx_.checkpoints[seg], dt, min(every, nsteps - seg * every), False)
             while steps:
                 Un, U1, U2 = steps.pop()

@@ -1,6 +1,7 @@
 """Order of the rollout's calls and what they are given, on a stand-in for the library's context whose
 step multiplies by 3/2: ragged and single segments, no steps, no gradient asked for."""
 import types
+import weakref
 
 import pytest
 
@@ -55,3 +56,30 @@ def test_rollout_without_a_gradient_keeps_no_stages():
         assert float(adjoint.rollout(c, U0, 0.1, 5, 2)[0]) == 1.5 ** 5
     adjoint.rollout(c, U0.detach(), 0.1, 5, 2)
     assert c.kept == 0
+
+
+def test_one_segment_is_kept_per_context():
+    """Rollouts that are chained in one graph, or whose backward pass never comes, hold the stages of
+    the latest one only; the others recompute theirs from the checkpoint, which stays."""
+    class Watched(Ctx):
+        def rk_step_stages(self, U, dt, U1, U2, nxt=None):
+            super().rk_step_stages(U, dt, U1, U2, nxt)
+            self.stages.append(weakref.ref(U1))
+
+        def alive(self):
+            return sum(r() is not None for r in self.stages)
+
+    c = Watched()
+    c.stages = []
+    waiting = adjoint.rollout(c, torch.ones(2, dtype=torch.float64, requires_grad=True), 0.1, 4, 4)
+    assert c.alive() == 4
+    U0 = torch.ones(2, dtype=torch.float64, requires_grad=True)
+    U = U0
+    for n in (3, 5, 2):
+        U = adjoint.rollout(c, U, 0.1, n, 4)
+    assert c.alive() == 2
+    U.sum().backward()
+    assert c.reversed_from == [1.5 ** i for i in reversed(range(10))]
+    waiting.sum().backward()
+    assert float(U0.grad[0]) == 1.5 ** 10 and c.reversed_from[10:] == [1.5 ** i for i in reversed(range(4))]
+    assert c.alive() == 0
