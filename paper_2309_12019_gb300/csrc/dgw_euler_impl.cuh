@@ -57,8 +57,9 @@ __device__ __forceinline__ void euler_flux(const EulerState& s, Real m, Real en,
 
 // Sensor of Sec. 4 (or the comparison sensor of Zhao et al., stab = ZHAO) of a 1D cell
 // with coefficients c from its face neighbours cn[0] (left) and cn[1] (right), where
-// they exist.
-template <int P>
+// they exist.  TILE: with the operations of process_tile from the weights on (roots and quotients
+// of full precision, the ratio itself against b), so that a scalar cell gets the same bits.
+template <int P, bool TILE = false>
 __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, const Real* c, const Real (*cn)[P + 1],
                                           const bool* has)
 {
@@ -93,7 +94,7 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
 #pragma unroll
         for (int k = 1; k < N1; ++k) dacc[k] = fma(wl, c[k] - cl[k], dacc[k]);
     }
-    const Real inv = div_w(Real(1), wsum);
+    const Real inv = (TILE && !kF32 && A.stab != STAB_ZHAO) ? Real(1) : div_w(Real(1), wsum);
     if (A.stab == STAB_ZHAO) {
         if (me == 0) return Real(0);
         const Real lin0 = Real(1) - Real(me) * A.w_nbr;
@@ -102,14 +103,31 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
         for (int f = 0; f < 2; ++f)
             if (has[f]) dev += zpow(A, fabs(wnb[f] * inv / A.w_nbr - Real(1)));
         const Real minlin = lin0 < A.w_nbr ? lin0 : A.w_nbr;
+        if (TILE) return dev / (zpow(A, fabs(Real(1) / minlin - Real(1))) + Real(me));
         return dev * rcp_e(zpow(A, fabs(rcp_e(minlin) - Real(1))) + Real(me));
+    }
+    dacc[0] = Real(0);
+    if constexpr (TILE) {
+        Real r, g;
+        if constexpr (kF32) {
+#pragma unroll
+            for (int k = 1; k < N1; ++k) dacc[k] *= inv;
+            const Real num = sqrt_r(fmax(qform<P>(T, dacc), Real(0)));
+            if (num <= A.eps_s) return Real(0);
+            if (beta0 <= Real(0)) return Real(1);
+            r = num / sqrt_r(beta0);
+            g = r < Real(1) ? r : Real(1);
+        } else {
+            g = sensor_ratio(qform<P>(T, dacc), beta0, wsum, A.eps_s, &r);
+        }
+        if (!A.q_one) g = pow(g, A.q);
+        return less_pos(r, A.b) ? Real(0) : g;
     }
     // U - U* = sum_l w_l (c - c_l); the ratio r = ||U - U*|| / ||U|| is taken through
     // its square: r <= 1 iff qd <= beta0, r < b iff r^2 < b^2, ||U - U*|| <= eps_s iff
     // qd <= eps_s^2
 #pragma unroll
     for (int k = 1; k < N1; ++k) dacc[k] *= inv;
-    dacc[0] = Real(0);
     const Real qd = fmax(qform<P>(T, dacc), Real(0));
     if (qd <= A.eps_s * A.eps_s) return Real(0);
     if (beta0 <= Real(0)) return Real(1);

@@ -11,8 +11,10 @@
 // volume term, which needs no neighbour, runs between the barrier's arrive and wait.
 //
 // CTAs are as small as the cluster limit lets them be, which spreads the FP64 work over the most
-// SMs.  The scheme and the order of its operations are those of process_tile and euler_kernel;
-// each face is evaluated by both of its cells from the same values in the same way.
+// SMs.  The scheme is that of process_tile and euler_kernel; a scalar cell on one lane also takes
+// their operations in their order, the sensor's included, and so their bits.  (Euler cells and cells
+// on eight lanes agree with the stage kernels to rounding.)  Each face is evaluated by both of its
+// cells from the same values in the same way.
 //
 // Double, up to kWideMax cells: eight lanes per cell.  A warp's FP64 instruction occupies its
 // scheduler's share of the FP64 pipe for 64 cycles however many lanes are active and however many
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const __grid_constan
                 nb[1][k] = w.has_r ? sc[buf][k][w.col + 1] : Real(0);
             }
             Real gamma = A.stab == STAB_LO ? Real(1) : Real(0);
-            if (A.stab >= STAB_WENO) gamma = sensor_1d<P>(A, T, c, nb, has);
+            if (A.stab >= STAB_WENO) gamma = sensor_1d<P, true>(A, T, c, nb, has);
             // fluxes of the left and right face; beyond a side the ghost of the boundary
             Real ul, ur, t, h[2];
             line_ends(nb[0], t, ul);
@@ -434,12 +436,12 @@ struct WideLane {
 // that one with its square root as one reciprocal square root: gamma = ||D|| / (W ||U||) for
 // D = sum_l w_l (c - c_l), W = sum_l w_l.  States whose products could leave the range of double
 // take sensor_1d.
-template <int P>
+template <int P, bool TILE>
 __device__ __forceinline__ Real wide_sensor(const KParams& A, const Tab<P>& T, const WideLane<P>& w, const Real (&c)[P + 1],
                                             const Real (&nb)[2][P + 1], const bool (&has)[2])
 {
     constexpr int N1 = P + 1;
-    if (A.stab == STAB_ZHAO) return sensor_1d<P>(A, T, c, nb, has);
+    if (A.stab == STAB_ZHAO) return sensor_1d<P, TILE>(A, T, c, nb, has);
     Real cl[N1];
 #pragma unroll
     for (int k = 0; k < N1; ++k) cl[k] = w.role == 1 ? nb[0][k] : (w.role == 2 ? nb[1][k] : c[k]);
@@ -475,7 +477,7 @@ __device__ __forceinline__ Real wide_sensor(const KParams& A, const Tab<P>& T, c
     const bool flat = !less_pos(Real(0), qd) || !less_pos(Real(0), beta0);
     if (!less_pos(hi, Real(1e24)) || !less_pos(Real(1e-16), lo) || !less_pos(Real(1e-16), d20) ||
         !(flat || less_pos(Real(1e-280), pr)))
-        return sensor_1d<P>(A, T, c, nb, has);
+        return sensor_1d<P, TILE>(A, T, c, nb, has);
     if (!less_pos((A.eps_s * A.eps_s) * W2, qd)) return Real(0);
     if (flat) return Real(1);
     Real r = Real(1);
@@ -546,7 +548,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
             nb[1][k] = w.has_r ? sc[buf][k][w.col + 1] : Real(0);
         }
         Real gamma = A.stab == STAB_LO ? Real(1) : Real(0);
-        if (A.stab >= STAB_WENO) gamma = wide_sensor<P>(A, T, g, c, nb, has);
+        if (A.stab >= STAB_WENO) gamma = wide_sensor<P, true>(A, T, g, c, nb, has);
         // the flux of the lane's face
         Real other;
         {
@@ -708,7 +710,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
             nb[1][k] = w.has_r ? S.sv[buf][k][w.col + 1] : Real(0);
         }
         Real gamma = A.stab == STAB_LO ? Real(1) : Real(0);
-        if (A.stab >= STAB_WENO) gamma = wide_sensor<P>(A, T, g, c[0], nb, has);
+        if (A.stab >= STAB_WENO) gamma = wide_sensor<P, false>(A, T, g, c[0], nb, has);
         // lane sub < 6: component sub >> 1 of face sub & 1, between columns col - 1 + side and
         // col + side; beyond a side the ghost: the inner end, its momentum mirrored at a wall
         {

@@ -134,7 +134,7 @@ static Real max_nan(Real a, Real b) { return a < b ? b : a; }
 static Real rsqrt(Real x) { return 1 / std::sqrt(x); }
 static Real fma_x(Real a, Real b, Real c) { return std::fma(a, b, c); }
 using std::fabs; using std::fma; using std::pow;
-template <int P> Real sensor_1d(const KParams&, const Tab<P>&, const Real* c, const Real (*n)[P + 1], const bool*) { return 0.5 + 0.1 * std::tanh(c[1] + n[0][1] - n[1][1]); }
+template <int P, bool TILE = false> Real sensor_1d(const KParams&, const Tab<P>&, const Real* c, const Real (*n)[P + 1], const bool*) { return 0.5 + 0.1 * std::tanh(c[1] + n[0][1] - n[1][1]); }
 template <int N1, int NQ> void interp_sym(const Real (&)[NQ][N1], const Real (&r)[N1], Real (&u)[NQ]) { for (auto& x : u) x = r[0]; }
 template <bool, int N1, int NQ> void project_sym(const Real (&)[NQ][N1], const Real (&f)[NQ], Real (&o)[N1]) { for (auto& x : o) x = f[0]; }
 template <int F> void vol_flux(const KParams&, Real u, Real, Real, Real& f, Real& fy, Real& k) { f = 0.5 * u * u; fy = 0; k = std::fabs(u); }
