@@ -193,9 +193,12 @@ dgw_status dgw_sensor(dgw_ctx* ctx, const void* U, double* gamma, void* stream);
 
 /* nsteps steps of the optimal SSP-RK3 scheme (Eq. ssp) with step dt, in place on U
  * (device, K*E).  Each stage recomputes the sensor from the stage state.  The stage
- * states live in the context's buffers.  Launch sequence is replayed from a CUDA graph
- * cached per (U, dt, nsteps, stream) unless the stream is being captured.  nsteps = 0
- * does nothing; a negative nsteps or a non-finite dt is DGW_EINVAL. */
+ * states live in the context's buffers, and the launches are replayed from a CUDA graph
+ * cached per (U, dt, nsteps, stream) unless the stream is being captured.  1D meshes that
+ * one thread-block cluster holds (4096 cells in float, 2048 in double) take up to 1024 steps
+ * in one launch, with the stage states in registers; there a stage's sensor agrees with
+ * dgw_sensor to rounding, elsewhere bit for bit.  nsteps = 0 does nothing; a negative nsteps
+ * or a non-finite dt is DGW_EINVAL. */
 dgw_status dgw_rk_step(dgw_ctx* ctx, void* U, double dt, int nsteps, void* stream);
 
 /* As dgw_rk_step for a state held in HOST memory: copies U_in (host, K*E elements,
@@ -269,9 +272,10 @@ dgw_status dgw_adjoint_step(dgw_ctx* ctx, const void* U_n, const void* lam_np1, 
 /* One SSP-RK3 step (Eq. ssp) from U that keeps its two stage states: U1 = U + dt L(U)
  * and U2 = 3/4 U + 1/4 (U1 + dt L(U1)) are written to the caller's arrays (device, K*E),
  * and U^{n+1} to U_next when it is not NULL (U_next may equal U; NULL skips the third
- * stage).  U1 and U2 must not overlap U, U_next or each other.  For checkpointed
- * gradients: the recomputation of a segment stores the stage states, and the reverse
- * step then takes them (dgw_adjoint_step_stages) instead of recomputing them. */
+ * stage).  The launches are dgw_rk_step's, so the states are its bits.  U1 and U2 must not
+ * overlap U, U_next or each other.  For checkpointed gradients: the recomputation of a
+ * segment stores the stage states, and the reverse step then takes them
+ * (dgw_adjoint_step_stages) instead of recomputing them. */
 dgw_status dgw_rk_step_stages(dgw_ctx* ctx, const void* U, double dt, void* U1, void* U2, void* U_next,
                               void* stream);
 

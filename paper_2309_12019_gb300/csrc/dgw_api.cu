@@ -506,12 +506,13 @@ static cudaError_t enqueue_steps_rk24(const dgw_ctx* c, void* U, double dt, int 
 
 // 1D meshes that fit one thread-block cluster take all their steps in one launch
 // (dgw_line_impl.cuh); nsteps = 0 asks whether c's does.
-static cudaError_t line_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
+static cudaError_t line_steps(const dgw_ctx* c, const void* Uin, void* U, void* U1, void* U2, double dt, int nsteps,
+                              cudaStream_t s)
 {
     if (c->mesh.dim != 1) return cudaErrorNotSupported;
     const StageArgs a = base_args(c);
-    return c->eb == 8 ? launch_line_f64_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s)
-                      : launch_line_f32_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s);
+    return c->eb == 8 ? launch_line_f64_d1(a, c->p, c->flux.kind, Uin, U, U1, U2, dt, nsteps, c->params.rk_order, s)
+                      : launch_line_f32_d1(a, c->p, c->flux.kind, Uin, U, U1, U2, dt, nsteps, c->params.rk_order, s);
 }
 
 // One SSP-RK3 step (Eq. ssp): U1 = U + dt L(U); U2 = 3/4 U + 1/4 (U1 + dt L(U1));
@@ -519,7 +520,7 @@ static cudaError_t line_steps(const dgw_ctx* c, void* U, double dt, int nsteps, 
 // reads U only at its own element there.  Other orders: enqueue_steps_rk24.
 static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
-    const cudaError_t le = line_steps(c, U, dt, nsteps, s);
+    const cudaError_t le = line_steps(c, U, U, nullptr, nullptr, dt, nsteps, s);
     if (le != cudaErrorNotSupported) return le;
     if (c->params.rk_order != 3) return enqueue_steps_rk24(c, U, dt, nsteps, s);
     StageArgs a = base_args(c);
@@ -544,6 +545,25 @@ static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nstep
         }
     }
     return cudaSuccess;
+}
+
+// One SSP-RK3 step from U that keeps its stage states; without U_next the third stage is left out.
+// The launches are those of dgw_rk_step, so the states have its bits.
+static cudaError_t enqueue_stages(const dgw_ctx* c, const void* U, double dt, void* U1, void* U2, void* U_next, cudaStream_t s)
+{
+    cudaError_t e = line_steps(c, U, U_next, U1, U2, dt, 1, s);
+    if (e != cudaErrorNotSupported) return e;
+    StageArgs a = base_args(c);
+    a.pdl = 1;
+    a.Uk = U; a.Un = nullptr; a.Uout = U1;
+    a.cn = 0.0; a.ck = 1.0; a.cl = dt;
+    if ((e = launch(c, a, 0, s)) != cudaSuccess) return e;
+    a.Uk = U1; a.Un = U; a.Uout = U2;
+    a.cn = 0.75; a.ck = 0.25; a.cl = 0.25 * dt;
+    if ((e = launch(c, a, 0, s)) != cudaSuccess || !U_next) return e;
+    a.Uk = U2; a.Un = U; a.Uout = U_next;
+    a.cn = 1.0 / 3.0; a.ck = 2.0 / 3.0; a.cl = 2.0 / 3.0 * dt;
+    return launch(c, a, 0, s);
 }
 
 static const int kGraphChunk = 16;
@@ -587,7 +607,7 @@ extern "C" dgw_status dgw_rk_step(dgw_ctx* c, void* U, double dt, int nsteps, vo
     cudaStream_t s = (cudaStream_t)stream;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (s != nullptr) DGW_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (s == nullptr || cap != cudaStreamCaptureStatusNone || line_steps(c, U, dt, 0, s) == cudaSuccess) {
+    if (s == nullptr || cap != cudaStreamCaptureStatusNone || line_steps(c, U, U, nullptr, nullptr, dt, 0, s) == cudaSuccess) {
         DGW_CUDA(enqueue_steps(c, U, dt, nsteps, s));
         return DGW_OK;
     }
@@ -1673,14 +1693,7 @@ extern "C" dgw_status dgw_adjoint_step(dgw_ctx* c, const void* U_n, const void* 
     st = adjoint_ready(c);
     if (st != DGW_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    StageArgs a = base_args(c);
-    a.pdl = 1;
-    a.Uk = U_n; a.Un = nullptr; a.Uout = c->S1;
-    a.cn = 0.0; a.ck = 1.0; a.cl = dt;
-    DGW_CUDA(launch(c, a, 0, s));
-    a.Uk = c->S1; a.Un = U_n; a.Uout = c->S2;
-    a.cn = 0.75; a.ck = 0.25; a.cl = 0.25 * dt;
-    DGW_CUDA(launch(c, a, 0, s));
+    DGW_CUDA(enqueue_stages(c, U_n, dt, c->S1, c->S2, nullptr, s));
     DGW_CUDA(vjp_combine(c, c->S2, lam_np1, lam_np1, 2.0 / 3.0, nullptr, 0.0, nullptr, 0.0, 2.0 / 3.0 * dt,
                          c->adj_b1, s));
     DGW_CUDA(vjp_combine(c, c->S1, c->adj_b1, c->adj_b1, 0.25, nullptr, 0.0, nullptr, 0.0, 0.25 * dt,
@@ -1703,19 +1716,7 @@ extern "C" dgw_status dgw_rk_step_stages(dgw_ctx* c, const void* U, double dt, v
     if (c->params.rk_order != 3) return fail(DGW_EUNSUPPORTED, "stage states of the SSP-RK3 step (rk_order 3)");
     if (c->state_sides) return fail(DGW_EUNSUPPORTED, "dgw_rk_step_stages keeps no time (prescribed-state sides)");
     cudaStream_t s = (cudaStream_t)stream;
-    StageArgs a = base_args(c);
-    a.pdl = 1;
-    a.Uk = U; a.Un = nullptr; a.Uout = U1;
-    a.cn = 0.0; a.ck = 1.0; a.cl = dt;
-    DGW_CUDA(launch(c, a, 0, s));
-    a.Uk = U1; a.Un = U; a.Uout = U2;
-    a.cn = 0.75; a.ck = 0.25; a.cl = 0.25 * dt;
-    DGW_CUDA(launch(c, a, 0, s));
-    if (U_next) {
-        a.Uk = U2; a.Un = U; a.Uout = U_next;
-        a.cn = 1.0 / 3.0; a.ck = 2.0 / 3.0; a.cl = 2.0 / 3.0 * dt;
-        DGW_CUDA(launch(c, a, 0, s));
-    }
+    DGW_CUDA(enqueue_stages(c, U, dt, U1, U2, U_next, s));
     return DGW_OK;
 }
 

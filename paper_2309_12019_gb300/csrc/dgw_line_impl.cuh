@@ -39,7 +39,9 @@ constexpr int kWideMax = kF32 ? 0 : kLineCluster * kWideCells;
 // cn Un + ck U + cl L(U); order 4 (ten stages): combination 0 nine times, with the register
 // recombination after the fifth, then combination 1.
 struct LineSteps {
-    Real* U;
+    const Real* Uin;
+    Real* U;                               // the state after the last step (may be Uin; null: not asked for)
+    Real* keep[2];                         // the states after stages 0 and 1 (both null: not asked for)
     int nsteps, order, stages, cells;      // cells: per CTA (all but the last are full)
     Real cn[3], ck[3], cl[3];
 };
@@ -140,10 +142,11 @@ __device__ __forceinline__ Real line_update(const KParams& A, const Tab<P>& T, i
     return fma(cn, un, fma(cl, Lk, ck * c[k]));
 }
 
-// Runs the stages of nsteps steps: stage(r, cn, ck, cl) advances c in place.
-template <int NC, class Stage>
-__device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real (&un)[NC], Stage&& stage)
+// Runs the stages of nsteps steps: stage(cn, ck, cl) advances c in place, store(U) writes it out.
+template <int NC, class Stage, class Store>
+__device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real (&un)[NC], Stage&& stage, Store&& store)
 {
+    const bool keep = L.keep[0] != nullptr;
     for (int n = 0; n < L.nsteps; ++n) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) un[k] = c[k];
@@ -151,6 +154,7 @@ __device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real
         for (int r = 0; r < L.stages; ++r) {
             const int i = L.order == 4 ? (r == 9) : r;
             stage(L.cn[i], L.ck[i], L.cl[i]);
+            if (keep && r < 2) store(r == 0 ? L.keep[0] : L.keep[1]);
             if (L.order == 4 && r == 4) {
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
@@ -160,6 +164,7 @@ __device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real
             }
         }
     }
+    if (L.U) store(L.U);
 }
 
 template <int P, int FLUX>
@@ -171,7 +176,7 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const __grid_constan
     const LinePlace w(A, L, threadIdx.x);
     Real c[N1], un[N1];
 #pragma unroll
-    for (int k = 0; k < N1; ++k) c[k] = w.in ? L.U[k * A.E + w.gx] : Real(0);
+    for (int k = 0; k < N1; ++k) c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(0);
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const Real xl = fma_x(Real(w.gx), A.h, A.x0), xr = fma_x(Real(w.gx + 1), A.h, A.x0);
     const Real xc = fma_x(Real(w.gx) + Real(0.5), A.h, A.x0);
@@ -235,11 +240,12 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const __grid_constan
             for (int k = 0; k < N1; ++k) c[k] = out[k];
         }
         buf ^= 1;
-    });
-    if (!w.in) return;
+    }, [&](Real* U) {
+        if (!w.in) return;
 #pragma unroll
-    for (int k = 0; k < N1; ++k) L.U[k * A.E + w.gx] = c[k];
-    if (chk != chk) atomicOr(A.flag, 1u);
+        for (int k = 0; k < N1; ++k) U[k * A.E + w.gx] = c[k];
+    });
+    if (w.in && chk != chk) atomicOr(A.flag, 1u);
 }
 
 // The Euler system: a cell publishes its density coefficients and, for each of its ends, the
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(kLineThreads) line_euler_kernel(const __grid_c
     const LinePlace w(A, L, threadIdx.x);
     Real c[3 * N1], un[3 * N1];
 #pragma unroll
-    for (int k = 0; k < 3 * N1; ++k) c[k] = w.in ? L.U[k * A.E + w.gx] : Real(k % N1 == 0 ? (k == N1 ? 0 : 1) : 0);
+    for (int k = 0; k < 3 * N1; ++k) c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(k % N1 == 0 ? (k == N1 ? 0 : 1) : 0);
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const bool has[2] = {w.has_l, w.has_r};
     Real chk = Real(0);
@@ -367,11 +373,12 @@ __global__ void __launch_bounds__(kLineThreads) line_euler_kernel(const __grid_c
                 }
         }
         buf ^= 1;
-    });
-    if (!w.in) return;
+    }, [&](Real* U) {
+        if (!w.in) return;
 #pragma unroll
-    for (int k = 0; k < 3 * N1; ++k) L.U[k * A.E + w.gx] = c[k];
-    if (chk != chk) atomicOr(A.flag, 1u);
+        for (int k = 0; k < 3 * N1; ++k) U[k * A.E + w.gx] = c[k];
+    });
+    if (w.in && chk != chk) atomicOr(A.flag, 1u);
 }
 
 // ------------------------------------------------------------------------------------
@@ -503,7 +510,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
     for (int k = 0; k < N1; ++k) {
         b[k] = T.B[q][k];
         a1[k] = k > 0 && km > 0 && ((km + k) & 1) == 0 ? T.A1[km][k] : Real(0);
-        c[k] = w.in ? L.U[k * A.E + w.gx] : Real(0);
+        c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(0);
     }
 #pragma unroll
     for (int i = 0; i < NQ; ++i) wd[i] = km > 0 ? T.WD[i][km] : Real(0);
@@ -577,10 +584,10 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
 #pragma unroll
         for (int k = 0; k < N1; ++k) c[k] = group_get(v[0], k);
         buf ^= 1;
+    }, [&](Real* U) {
+        if (owner) U[km * A.E + w.gx] = v[0];
     });
-    if (!owner) return;
-    L.U[km * A.E + w.gx] = v[0];
-    if (bad) atomicOr(A.flag, 1u);
+    if (owner && bad) atomicOr(A.flag, 1u);
 }
 
 // The Euler system, eight lanes per cell: a Gauss point or an end of the cell per lane, a
@@ -617,7 +624,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
 #pragma unroll
     for (int q = 0; q < 3; ++q)
 #pragma unroll
-        for (int k = 0; k < N1; ++k) c[q][k] = w.in ? L.U[(q * N1 + k) * A.E + w.gx] : Real(k == 0 && q != 1 ? 1 : 0);
+        for (int k = 0; k < N1; ++k) c[q][k] = w.in ? L.Uin[(q * N1 + k) * A.E + w.gx] : Real(k == 0 && q != 1 ? 1 : 0);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = g.sub + 8 * r < NM ? g.sub + 8 * r : NM - 1;
@@ -630,7 +637,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
 #pragma unroll
         for (int m = 0; m < N1; ++m) a1[r][m] = m > 0 && mdeg[r] > 0 && ((mdeg[r] + m) & 1) == 0 ? T.A1[mdeg[r]][m] : Real(0);
         // (lanes without a cell keep a state at rest: no divisions by zero, which are slow)
-        v[r] = w.in ? L.U[mode[r] * A.E + w.gx] : Real(mdeg[r] == 0 && mcomp[r] != 1 ? 1 : 0);
+        v[r] = w.in ? L.Uin[mode[r] * A.E + w.gx] : Real(mdeg[r] == 0 && mcomp[r] != 1 ? 1 : 0);
     }
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const bool has[2] = {w.has_l, w.has_r};
@@ -751,12 +758,13 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
         }
         __syncwarp();          // the next stage's modes replace those that other lanes read above
         buf ^= 1;
-    });
-    if (!w.in) return;
+    }, [&](Real* U) {
+        if (!w.in) return;
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (g.sub + 8 * r < NM) L.U[mode[r] * A.E + w.gx] = v[r];
-    if (bad) atomicOr(A.flag, 1u);
+        for (int r = 0; r < R; ++r)
+            if (g.sub + 8 * r < NM) U[mode[r] * A.E + w.gx] = v[r];
+    });
+    if (w.in && bad) atomicOr(A.flag, 1u);
 }
 
 // Largest cluster of `fn` on the current device with `threads` threads a CTA: 16, 8, or 0 if
@@ -865,17 +873,22 @@ static cudaError_t launch_line_p(const KParams& a, LineSteps& L, int flux, bool 
     }
 }
 
-// nsteps steps of the mesh of s in place on U, or (nsteps = 0) only whether the mesh fits.
+// nsteps steps of the mesh of s from Uin to U, or (nsteps = 0) only whether the mesh fits.  One step may
+// keep the states of its first two stages (U1, U2); without U it then ends with them.
 // cudaErrorNotSupported: it does not fit one cluster, nothing was launched.
-static cudaError_t launch_line(const StageArgs& s, int p, int flux, void* U, double dt, int nsteps, int order, cudaStream_t st)
+static cudaError_t launch_line(const StageArgs& s, int p, int flux, const void* Uin, void* U, void* U1, void* U2, double dt,
+                               int nsteps, int order, cudaStream_t st)
 {
     if (s.nx > kLineCluster * kLineThreads) return cudaErrorNotSupported;
     const KParams a = make_params(s);
     LineSteps L;
     memset(&L, 0, sizeof L);
+    L.Uin = static_cast<const Real*>(Uin);
     L.U = static_cast<Real*>(U);
+    L.keep[0] = static_cast<Real*>(U1);
+    L.keep[1] = static_cast<Real*>(U2);
     L.order = order;
-    L.stages = order == 4 ? 10 : order;
+    L.stages = order == 4 ? 10 : (U ? order : 2);
     const double t3[3][3] = {{0.0, 1.0, 1.0}, {0.75, 0.25, 0.25}, {1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0}};
     const double t2[2][3] = {{0.0, 1.0, 1.0}, {0.5, 0.5, 0.5}};
     const double t4[2][3] = {{0.0, 1.0, 1.0 / 6.0}, {1.0, 3.0 / 5.0, 1.0 / 10.0}};
@@ -896,6 +909,7 @@ static cudaError_t launch_line(const StageArgs& s, int p, int flux, void* U, dou
         else if (p == 2) e = launch_line_p<2>(a, L, flux, query, st);
         else if (p == 3) e = launch_line_p<3>(a, L, flux, query, st);
         if (e != cudaSuccess) return e;
+        L.Uin = L.U;
         left -= L.nsteps;
     } while (left > 0);
     return cudaSuccess;

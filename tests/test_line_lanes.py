@@ -24,7 +24,7 @@ template <class K> static int differ(K kernel, int nc, int order, int bc)
         A.stab = STAB_WENO; A.nx = cells; A.E = cells; A.flag = &flag;
         for (int& b : A.bc) b = bc;
         LineSteps L = {};
-        L.U = U[up].data(); L.nsteps = 2; L.order = order; L.stages = order == 4 ? 10 : order; L.cells = cells;
+        L.Uin = L.U = U[up].data(); L.nsteps = 2; L.order = order; L.stages = order == 4 ? 10 : order; L.cells = cells;
         for (int i = 0; i < 3; ++i) { L.cn[i] = 0.3 * i; L.ck[i] = 1.0 - 0.3 * i; L.cl[i] = 1e-3; }
         run_lanes(8 * cells, up == 1, [&] { kernel(A, L); });
     }
