@@ -506,13 +506,12 @@ static cudaError_t enqueue_steps_rk24(const dgw_ctx* c, void* U, double dt, int 
 
 // 1D meshes that fit one thread-block cluster take all their steps in one launch
 // (dgw_line_impl.cuh); nsteps = 0 asks whether c's does.
-static cudaError_t line_steps(const dgw_ctx* c, const void* Uin, void* U, void* U1, void* U2, double dt, int nsteps,
-                              cudaStream_t s)
+static cudaError_t line_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
     if (c->mesh.dim != 1) return cudaErrorNotSupported;
     const StageArgs a = base_args(c);
-    return c->eb == 8 ? launch_line_f64_d1(a, c->p, c->flux.kind, Uin, U, U1, U2, dt, nsteps, c->params.rk_order, s)
-                      : launch_line_f32_d1(a, c->p, c->flux.kind, Uin, U, U1, U2, dt, nsteps, c->params.rk_order, s);
+    return c->eb == 8 ? launch_line_f64_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s)
+                      : launch_line_f32_d1(a, c->p, c->flux.kind, U, dt, nsteps, c->params.rk_order, s);
 }
 
 // One SSP-RK3 step (Eq. ssp): U1 = U + dt L(U); U2 = 3/4 U + 1/4 (U1 + dt L(U1));
@@ -520,7 +519,7 @@ static cudaError_t line_steps(const dgw_ctx* c, const void* Uin, void* U, void* 
 // reads U only at its own element there.  Other orders: enqueue_steps_rk24.
 static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
-    const cudaError_t le = line_steps(c, U, U, nullptr, nullptr, dt, nsteps, s);
+    const cudaError_t le = line_steps(c, U, dt, nsteps, s);
     if (le != cudaErrorNotSupported) return le;
     if (c->params.rk_order != 3) return enqueue_steps_rk24(c, U, dt, nsteps, s);
     StageArgs a = base_args(c);
@@ -548,22 +547,25 @@ static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nstep
 }
 
 // One SSP-RK3 step from U that keeps its stage states; without U_next the third stage is left out.
-// The launches are those of dgw_rk_step, so the states have its bits.
+// By the kernels of enqueue_steps, so the states have dgw_rk_step's bits.
 static cudaError_t enqueue_stages(const dgw_ctx* c, const void* U, double dt, void* U1, void* U2, void* U_next, cudaStream_t s)
 {
-    cudaError_t e = line_steps(c, U, U_next, U1, U2, dt, 1, s);
-    if (e != cudaErrorNotSupported) return e;
     StageArgs a = base_args(c);
     a.pdl = 1;
-    a.Uk = U; a.Un = nullptr; a.Uout = U1;
-    a.cn = 0.0; a.ck = 1.0; a.cl = dt;
-    if ((e = launch(c, a, 0, s)) != cudaSuccess) return e;
-    a.Uk = U1; a.Un = U; a.Uout = U2;
-    a.cn = 0.75; a.ck = 0.25; a.cl = 0.25 * dt;
-    if ((e = launch(c, a, 0, s)) != cudaSuccess || !U_next) return e;
-    a.Uk = U2; a.Un = U; a.Uout = U_next;
-    a.cn = 1.0 / 3.0; a.ck = 2.0 / 3.0; a.cl = 2.0 / 3.0 * dt;
-    return launch(c, a, 0, s);
+    auto stage = [&](const void* Uk, const void* Un, void* Uout, double cn, double ck, double cl) {
+        a.Uk = Uk; a.Un = Un; a.Uout = Uout;
+        a.cn = cn; a.ck = ck; a.cl = cl;
+        if (c->mesh.dim == 1) {
+            const cudaError_t e = c->eb == 8 ? launch_line_stage_f64_d1(a, c->p, c->flux.kind, s)
+                                             : launch_line_stage_f32_d1(a, c->p, c->flux.kind, s);
+            if (e != cudaErrorNotSupported) return e;
+        }
+        return launch(c, a, 0, s);
+    };
+    cudaError_t e = stage(U, nullptr, U1, 0.0, 1.0, dt);
+    if (e == cudaSuccess) e = stage(U1, U, U2, 0.75, 0.25, 0.25 * dt);
+    if (e == cudaSuccess && U_next) e = stage(U2, U, U_next, 1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0 * dt);
+    return e;
 }
 
 static const int kGraphChunk = 16;
@@ -607,7 +609,7 @@ extern "C" dgw_status dgw_rk_step(dgw_ctx* c, void* U, double dt, int nsteps, vo
     cudaStream_t s = (cudaStream_t)stream;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (s != nullptr) DGW_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (s == nullptr || cap != cudaStreamCaptureStatusNone || line_steps(c, U, U, nullptr, nullptr, dt, 0, s) == cudaSuccess) {
+    if (s == nullptr || cap != cudaStreamCaptureStatusNone || line_steps(c, U, dt, 0, s) == cudaSuccess) {
         DGW_CUDA(enqueue_steps(c, U, dt, nsteps, s));
         return DGW_OK;
     }

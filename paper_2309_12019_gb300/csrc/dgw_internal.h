@@ -150,14 +150,13 @@ cudaError_t launch_stage_f64_d1(const StageArgs& a, int p, int flux, int mode, c
 cudaError_t launch_stage_f64_d2(const StageArgs& a, int p, int flux, int mode, cudaStream_t s);
 
 // nsteps Runge-Kutta steps of a 1D mesh that fits one thread-block cluster, in one launch per
-// 1024 steps, from Uin to U (which may be the same); cudaErrorNotSupported (nothing launched) where
-// the mesh does not fit.  nsteps = 0 only asks.  One step of order 3 may keep the states of its first
-// two stages in U1 and U2 (else null), and without U does not take its third.  Of a: the mesh,
-// flux, stabilization and flag.
-cudaError_t launch_line_f32_d1(const StageArgs& a, int p, int flux, const void* Uin, void* U, void* U1, void* U2, double dt,
-                               int nsteps, int order, cudaStream_t s);
-cudaError_t launch_line_f64_d1(const StageArgs& a, int p, int flux, const void* Uin, void* U, void* U1, void* U2, double dt,
-                               int nsteps, int order, cudaStream_t s);
+// 1024 steps, in place on U; cudaErrorNotSupported (nothing launched) where the mesh does not
+// fit.  nsteps = 0 only asks.  Of a: the mesh, flux, stabilization and flag.  launch_line_stage_*: the
+// one stage of a by the same kernels, which has the bits of that stage of a step.
+cudaError_t launch_line_f32_d1(const StageArgs& a, int p, int flux, void* U, double dt, int nsteps, int order, cudaStream_t s);
+cudaError_t launch_line_f64_d1(const StageArgs& a, int p, int flux, void* U, double dt, int nsteps, int order, cudaStream_t s);
+cudaError_t launch_line_stage_f32_d1(const StageArgs& a, int p, int flux, cudaStream_t s);
+cudaError_t launch_line_stage_f64_d1(const StageArgs& a, int p, int flux, cudaStream_t s);
 
 // Batch kernels per (degree p, tile height `rows`): 2D float tiles of 2, 4 or 8 cell rows,
 // 2D double tiles of kTileY2, 1D tiles of one row (batch_rows_built_*).

@@ -40,8 +40,8 @@ constexpr int kWideMax = kF32 ? 0 : kLineCluster * kWideCells;
 // recombination after the fifth, then combination 1.
 struct LineSteps {
     const Real* Uin;
-    Real* U;                               // the state after the last step (may be Uin; null: not asked for)
-    Real* keep[2];                         // the states after stages 0 and 1 (both null: not asked for)
+    const Real* Un;                        // start state of the step, if not Uin (a single later stage; else null)
+    Real* U;                               // the result (may be Uin or Un)
     int nsteps, order, stages, cells;      // cells: per CTA (all but the last are full)
     Real cn[3], ck[3], cl[3];
 };
@@ -142,19 +142,19 @@ __device__ __forceinline__ Real line_update(const KParams& A, const Tab<P>& T, i
     return fma(cn, un, fma(cl, Lk, ck * c[k]));
 }
 
-// Runs the stages of nsteps steps: stage(cn, ck, cl) advances c in place, store(U) writes it out.
-template <int NC, class Stage, class Store>
-__device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real (&un)[NC], Stage&& stage, Store&& store)
+// Runs the stages of nsteps steps: stage(cn, ck, cl) advances c in place.
+template <int NC, class Stage>
+__device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real (&un)[NC], Stage&& stage)
 {
-    const bool keep = L.keep[0] != nullptr;
     for (int n = 0; n < L.nsteps; ++n) {
+        if (!L.Un) {
 #pragma unroll
-        for (int k = 0; k < NC; ++k) un[k] = c[k];
+            for (int k = 0; k < NC; ++k) un[k] = c[k];
+        }
 #pragma unroll 1
         for (int r = 0; r < L.stages; ++r) {
             const int i = L.order == 4 ? (r == 9) : r;
             stage(L.cn[i], L.ck[i], L.cl[i]);
-            if (keep && r < 2) store(r == 0 ? L.keep[0] : L.keep[1]);
             if (L.order == 4 && r == 4) {
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
@@ -164,7 +164,6 @@ __device__ __forceinline__ void line_run(const LineSteps& L, Real (&c)[NC], Real
             }
         }
     }
-    if (L.U) store(L.U);
 }
 
 template <int P, int FLUX>
@@ -176,7 +175,10 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const __grid_constan
     const LinePlace w(A, L, threadIdx.x);
     Real c[N1], un[N1];
 #pragma unroll
-    for (int k = 0; k < N1; ++k) c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(0);
+    for (int k = 0; k < N1; ++k) {
+        c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(0);
+        un[k] = w.in && L.Un ? L.Un[k * A.E + w.gx] : c[k];
+    }
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const Real xl = fma_x(Real(w.gx), A.h, A.x0), xr = fma_x(Real(w.gx + 1), A.h, A.x0);
     const Real xc = fma_x(Real(w.gx) + Real(0.5), A.h, A.x0);
@@ -240,12 +242,11 @@ __global__ void __launch_bounds__(kLineThreads) line_kernel(const __grid_constan
             for (int k = 0; k < N1; ++k) c[k] = out[k];
         }
         buf ^= 1;
-    }, [&](Real* U) {
-        if (!w.in) return;
-#pragma unroll
-        for (int k = 0; k < N1; ++k) U[k * A.E + w.gx] = c[k];
     });
-    if (w.in && chk != chk) atomicOr(A.flag, 1u);
+    if (!w.in) return;
+#pragma unroll
+    for (int k = 0; k < N1; ++k) L.U[k * A.E + w.gx] = c[k];
+    if (chk != chk) atomicOr(A.flag, 1u);
 }
 
 // The Euler system: a cell publishes its density coefficients and, for each of its ends, the
@@ -262,7 +263,10 @@ __global__ void __launch_bounds__(kLineThreads) line_euler_kernel(const __grid_c
     const LinePlace w(A, L, threadIdx.x);
     Real c[3 * N1], un[3 * N1];
 #pragma unroll
-    for (int k = 0; k < 3 * N1; ++k) c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(k % N1 == 0 ? (k == N1 ? 0 : 1) : 0);
+    for (int k = 0; k < 3 * N1; ++k) {
+        c[k] = w.in ? L.Uin[k * A.E + w.gx] : Real(k % N1 == 0 ? (k == N1 ? 0 : 1) : 0);
+        un[k] = w.in && L.Un ? L.Un[k * A.E + w.gx] : c[k];
+    }
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const bool has[2] = {w.has_l, w.has_r};
     Real chk = Real(0);
@@ -373,12 +377,11 @@ __global__ void __launch_bounds__(kLineThreads) line_euler_kernel(const __grid_c
                 }
         }
         buf ^= 1;
-    }, [&](Real* U) {
-        if (!w.in) return;
-#pragma unroll
-        for (int k = 0; k < 3 * N1; ++k) U[k * A.E + w.gx] = c[k];
     });
-    if (w.in && chk != chk) atomicOr(A.flag, 1u);
+    if (!w.in) return;
+#pragma unroll
+    for (int k = 0; k < 3 * N1; ++k) L.U[k * A.E + w.gx] = c[k];
+    if (chk != chk) atomicOr(A.flag, 1u);
 }
 
 // ------------------------------------------------------------------------------------
@@ -505,7 +508,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
     const WideLane<P> g(A, T, w, threadIdx.x & 7);
     const int q = g.sub < NQ ? g.sub : NQ - 1, km = g.sub < N1 ? g.sub : P;
     const bool owner = w.in && g.sub < N1;
-    Real b[N1], wd[NQ], a1[N1], c[N1], v[1], un[1] = {Real(0)};
+    Real b[N1], wd[NQ], a1[N1], c[N1], v[1], un[1];
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
         b[k] = T.B[q][k];
@@ -518,6 +521,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
 #pragma unroll
     for (int k = 1; k < N1; ++k)
         if (km == k) v[0] = c[k];
+    un[0] = owner && L.Un ? L.Un[km * A.E + w.gx] : v[0];
     const Real sgk = (km & 1) ? Real(-1) : Real(1), mk = A.two_h * T.minv[km];
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const Real xq = fma_x(A.hh, T.g[q], fma_x(Real(w.gx) + Real(0.5), A.h, A.x0));
@@ -584,10 +588,10 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_kernel(const __grid_
 #pragma unroll
         for (int k = 0; k < N1; ++k) c[k] = group_get(v[0], k);
         buf ^= 1;
-    }, [&](Real* U) {
-        if (owner) U[km * A.E + w.gx] = v[0];
     });
-    if (owner && bad) atomicOr(A.flag, 1u);
+    if (!owner) return;
+    L.U[km * A.E + w.gx] = v[0];
+    if (bad) atomicOr(A.flag, 1u);
 }
 
 // The Euler system, eight lanes per cell: a Gauss point or an end of the cell per lane, a
@@ -638,6 +642,7 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
         for (int m = 0; m < N1; ++m) a1[r][m] = m > 0 && mdeg[r] > 0 && ((mdeg[r] + m) & 1) == 0 ? T.A1[mdeg[r]][m] : Real(0);
         // (lanes without a cell keep a state at rest: no divisions by zero, which are slow)
         v[r] = w.in ? L.Uin[mode[r] * A.E + w.gx] : Real(mdeg[r] == 0 && mcomp[r] != 1 ? 1 : 0);
+        un[r] = w.in && L.Un ? L.Un[mode[r] * A.E + w.gx] : v[r];
     }
     const bool find_lam = A.stab != STAB_DG && !A.lam_fixed;
     const bool has[2] = {w.has_l, w.has_r};
@@ -758,13 +763,12 @@ __global__ void __launch_bounds__(8 * kWideCells) line_wide_euler_kernel(const _
         }
         __syncwarp();          // the next stage's modes replace those that other lanes read above
         buf ^= 1;
-    }, [&](Real* U) {
-        if (!w.in) return;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (g.sub + 8 * r < NM) U[mode[r] * A.E + w.gx] = v[r];
     });
-    if (w.in && bad) atomicOr(A.flag, 1u);
+    if (!w.in) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (g.sub + 8 * r < NM) L.U[mode[r] * A.E + w.gx] = v[r];
+    if (bad) atomicOr(A.flag, 1u);
 }
 
 // Largest cluster of `fn` on the current device with `threads` threads a CTA: 16, 8, or 0 if
@@ -873,22 +877,44 @@ static cudaError_t launch_line_p(const KParams& a, LineSteps& L, int flux, bool 
     }
 }
 
-// nsteps steps of the mesh of s from Uin to U, or (nsteps = 0) only whether the mesh fits.  One step may
-// keep the states of its first two stages (U1, U2); without U it then ends with them.
-// cudaErrorNotSupported: it does not fit one cluster, nothing was launched.
-static cudaError_t launch_line(const StageArgs& s, int p, int flux, const void* Uin, void* U, void* U1, void* U2, double dt,
-                               int nsteps, int order, cudaStream_t st)
+// Launches L, whose nsteps may be 0 to ask whether the mesh fits.
+static cudaError_t launch_line_any(const KParams& a, LineSteps& L, int p, int flux, cudaStream_t st)
 {
-    if (s.nx > kLineCluster * kLineThreads) return cudaErrorNotSupported;
+    const bool query = L.nsteps == 0;
+    if (a.nx > kLineCluster * kLineThreads) return cudaErrorNotSupported;
+    if (p == 1) return launch_line_p<1>(a, L, flux, query, st);
+    if (p == 2) return launch_line_p<2>(a, L, flux, query, st);
+    if (p == 3) return launch_line_p<3>(a, L, flux, query, st);
+    return cudaErrorInvalidValue;
+}
+
+// The stage Uout = cn Un + ck Uk + cl L(Uk) of s alone.  cudaErrorNotSupported: the mesh does not
+// fit one cluster, nothing was launched.
+static cudaError_t launch_line_stage(const StageArgs& s, int p, int flux, cudaStream_t st)
+{
     const KParams a = make_params(s);
     LineSteps L;
     memset(&L, 0, sizeof L);
-    L.Uin = static_cast<const Real*>(Uin);
-    L.U = static_cast<Real*>(U);
-    L.keep[0] = static_cast<Real*>(U1);
-    L.keep[1] = static_cast<Real*>(U2);
+    L.Uin = a.Uk;
+    L.Un = a.has_un ? a.Un : nullptr;
+    L.U = a.Uout;
+    L.nsteps = L.stages = 1;
+    L.cn[0] = a.cn;
+    L.ck[0] = a.ck;
+    L.cl[0] = a.cl;
+    return launch_line_any(a, L, p, flux, st);
+}
+
+// nsteps steps of the mesh of s in place on U, or (nsteps = 0) only whether the mesh fits.
+// cudaErrorNotSupported: it does not fit one cluster, nothing was launched.
+static cudaError_t launch_line(const StageArgs& s, int p, int flux, void* U, double dt, int nsteps, int order, cudaStream_t st)
+{
+    const KParams a = make_params(s);
+    LineSteps L;
+    memset(&L, 0, sizeof L);
+    L.Uin = L.U = static_cast<Real*>(U);
     L.order = order;
-    L.stages = order == 4 ? 10 : (U ? order : 2);
+    L.stages = order == 4 ? 10 : order;
     const double t3[3][3] = {{0.0, 1.0, 1.0}, {0.75, 0.25, 0.25}, {1.0 / 3.0, 2.0 / 3.0, 2.0 / 3.0}};
     const double t2[2][3] = {{0.0, 1.0, 1.0}, {0.5, 0.5, 0.5}};
     const double t4[2][3] = {{0.0, 1.0, 1.0 / 6.0}, {1.0, 3.0 / 5.0, 1.0 / 10.0}};
@@ -903,13 +929,8 @@ static cudaError_t launch_line(const StageArgs& s, int p, int flux, const void* 
     int left = nsteps;
     do {
         L.nsteps = left < kChunk ? left : kChunk;
-        const bool query = nsteps == 0;
-        cudaError_t e = cudaErrorInvalidValue;
-        if (p == 1) e = launch_line_p<1>(a, L, flux, query, st);
-        else if (p == 2) e = launch_line_p<2>(a, L, flux, query, st);
-        else if (p == 3) e = launch_line_p<3>(a, L, flux, query, st);
+        const cudaError_t e = launch_line_any(a, L, p, flux, st);
         if (e != cudaSuccess) return e;
-        L.Uin = L.U;
         left -= L.nsteps;
     } while (left > 0);
     return cudaSuccess;

@@ -9,10 +9,13 @@ cudaError_t launch_stage_f32_d1(const StageArgs& a, int p, int flux, int mode, c
 {
     return f32_d1::launch(a, p, flux, mode, s);
 }
-cudaError_t launch_line_f32_d1(const StageArgs& a, int p, int flux, const void* Uin, void* U, void* U1, void* U2, double dt,
-                               int nsteps, int order, cudaStream_t s)
+cudaError_t launch_line_f32_d1(const StageArgs& a, int p, int flux, void* U, double dt, int nsteps, int order, cudaStream_t s)
 {
-    return f32_d1::launch_line(a, p, flux, Uin, U, U1, U2, dt, nsteps, order, s);
+    return f32_d1::launch_line(a, p, flux, U, dt, nsteps, order, s);
+}
+cudaError_t launch_line_stage_f32_d1(const StageArgs& a, int p, int flux, cudaStream_t s)
+{
+    return f32_d1::launch_line_stage(a, p, flux, s);
 }
 cudaError_t launch_batch_f32_d1(const BatchArgs& a, int p, int rows, int grid, cudaStream_t s)
 {
