@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(128, P <= 2 ? 4 : 1) vjp_kernel(const KParams 
     constexpr int N1 = P + 1, NQ = P + 2, K = Tab<P>::K, NF = 2 * DIM;
     constexpr int TN = DIM == 1 ? 1 : N1, NFQ = DIM == 1 ? 1 : NQ;
     const Tab<P>& T = tab<P>();
-    pdl_begin();
+    pdl_begin<kF32>();
     const int64_t E = A.E;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= E) return;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(128) gather_kernel(const int64_t E, const int 
                                                      Real* out)
 {
     constexpr int K = Tab<P>::K, NF = 2 * DIM;
-    pdl_begin();
+    pdl_begin<kF32>();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= E) return;
     const int ix = (int)(e % nx), iy = DIM == 2 ? (int)(e / nx) : 0;

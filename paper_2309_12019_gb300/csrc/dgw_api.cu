@@ -373,6 +373,14 @@ static StageArgs base_args(const dgw_ctx* c)
     return a;
 }
 
+// How a sequence of stages on s may overlap its launches (StageArgs.pdl)
+static int pdl_mode(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s == nullptr || cudaStreamIsCapturing(s, &cap) != cudaSuccess) return kPdlDirect;
+    return cap == cudaStreamCaptureStatusNone ? kPdlDirect : kPdlCaptured;
+}
+
 // t += dt on the device, after each step of a context with prescribed-state sides
 __global__ void advance_time_kernel(double* t, double dt) { *t += dt; }
 
@@ -460,7 +468,7 @@ __global__ void rk4_mix_kernel(Real* __restrict__ q2, Real* __restrict__ q1, int
 static cudaError_t enqueue_steps_rk24(const dgw_ctx* c, void* U, double dt, int nsteps, cudaStream_t s)
 {
     StageArgs a = base_args(c);
-    a.pdl = 1;
+    a.pdl = pdl_mode(s);
     for (int n = 0; n < nsteps; ++n) {
         if (c->params.rk_order == 2) {
             a.Uk = U; a.Un = nullptr; a.Uout = c->S1;
@@ -523,7 +531,7 @@ static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nstep
     if (le != cudaErrorNotSupported) return le;
     if (c->params.rk_order != 3) return enqueue_steps_rk24(c, U, dt, nsteps, s);
     StageArgs a = base_args(c);
-    a.pdl = 1;
+    a.pdl = pdl_mode(s);
     for (int n = 0; n < nsteps; ++n) {
         a.Uk = U; a.Un = nullptr; a.Uout = c->S1;
         a.cn = 0.0; a.ck = 1.0; a.cl = dt; a.t_off = 0.0;
@@ -551,7 +559,7 @@ static cudaError_t enqueue_steps(const dgw_ctx* c, void* U, double dt, int nstep
 static cudaError_t enqueue_stages(const dgw_ctx* c, const void* U, double dt, void* U1, void* U2, void* U_next, cudaStream_t s)
 {
     StageArgs a = base_args(c);
-    a.pdl = 1;
+    a.pdl = pdl_mode(s);
     auto stage = [&](const void* Uk, const void* Un, void* Uout, double cn, double ck, double cl) {
         a.Uk = Uk; a.Un = Un; a.Uout = Uout;
         a.cn = cn; a.ck = ck; a.cl = cl;
@@ -1644,9 +1652,9 @@ static cudaError_t vjp_combine(const dgw_ctx* c, const void* U, const void* lam,
                                cudaStream_t s)
 {
     StageArgs a = base_args(c);
-    a.pdl = 1;
-    a.Uk = U;
     const bool f64 = c->params.prec == DGW_FP64;
+    a.pdl = f64 ? kPdlCaptured : pdl_mode(s);
+    a.Uk = U;
     const int d = c->mesh.dim;
     cudaError_t e = f64 ? (d == 1 ? launch_vjp_f64_d1(a, c->p, c->flux.kind, lam, c->adj_ws, c->adj_wn, s)
                                   : launch_vjp_f64_d2(a, c->p, c->flux.kind, lam, c->adj_ws, c->adj_wn, s))
@@ -1661,7 +1669,7 @@ static cudaError_t vjp_combine(const dgw_ctx* c, const void* U, const void* lam,
     g.coef[0] = c0; g.coef[1] = c1; g.coef[2] = c2;
     g.cvjp = cv;
     g.out = out;
-    g.pdl = 1;
+    g.pdl = a.pdl;
     return f64 ? (d == 1 ? launch_gather_f64_d1(g, c->p, s) : launch_gather_f64_d2(g, c->p, s))
                : (d == 1 ? launch_gather_f32_d1(g, c->p, s) : launch_gather_f32_d2(g, c->p, s));
 }

@@ -486,7 +486,7 @@ static cudaError_t launch_euler2d_p(const StageArgs& s, int mode, cudaStream_t s
     KParams a = make_params(s);
     // (states that L2 holds are not asked for ahead: the triple point's 50 MB gain nothing)
     a.round_tiles = kF32 && (double)s.E * 4 * Tab<P>::K * sizeof(Real) > 64e6 ? euler2_blocks<P>() * sm_count() : 0;
-    constexpr int EY = euler2_rows<P>(), ENT = EX * EY;
+    constexpr int EY = euler2_rows<P>();
     dim3 grid((s.nx + EX - 1) / EX, (s.ny + EY - 1) / EY);
     if (grid.x == 0 || grid.y == 0) return cudaSuccess;
     const size_t smem = sizeof(Euler2Smem<P>);
@@ -494,11 +494,12 @@ static cudaError_t launch_euler2d_p(const StageArgs& s, int mode, cudaStream_t s
     const int dev = cur_device();
     if (!opted[dev][mode]) {
         const void* fn = mode == 0 ? (const void*)euler2d_kernel<P, 0> : (const void*)euler2d_kernel<P, 1>;
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemCta);
         if (e != cudaSuccess) return e;
         opted[dev][mode] = true;
     }
-    return launch_k(mode == 0 ? euler2d_kernel<P, 0> : euler2d_kernel<P, 1>, grid, ENT, smem, s.pdl != 0, st, a);
+    return mode == 0 ? launch_k<euler2d_kernel<P, 0>, true>(grid, EX * EY, smem, s.pdl, st, a)
+                     : launch_k<euler2d_kernel<P, 1>, true>(grid, EX * EY, smem, s.pdl, st, a);
 }
 
 static cudaError_t launch_euler2d(const StageArgs& s, int p, int mode, cudaStream_t st)

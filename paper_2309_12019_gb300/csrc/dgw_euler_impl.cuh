@@ -394,7 +394,7 @@ static cudaError_t launch_euler_p(const StageArgs& s, int mode, cudaStream_t st)
     const KParams a = make_params(s);
     const unsigned grid = (unsigned)((s.nx + TX - 1) / TX);
     if (grid == 0) return cudaSuccess;
-    return launch_k(mode == 0 ? euler_kernel<P, 0> : euler_kernel<P, 1>, grid, TX, 0, s.pdl != 0, st, a);
+    return mode == 0 ? launch_k<euler_kernel<P, 0>>(grid, TX, 0, s.pdl, st, a) : launch_k<euler_kernel<P, 1>>(grid, TX, 0, s.pdl, st, a);
 }
 
 static cudaError_t launch_euler(const StageArgs& s, int p, int mode, cudaStream_t st)

@@ -55,6 +55,8 @@ struct HostTables {
 void build_tables(int p, HostTables* t);
 void gauss_rule_public(int n, double* x, double* w);
 
+constexpr int kPdlDirect = 1, kPdlCaptured = 2;
+
 // Arguments of one stage launch: Uout = cn*Un + ck*Uk + cl*L(Uk), where L is the
 // stabilized DG right-hand side of Uk.  Pointers are of the kernel precision.
 struct StageArgs {
@@ -80,8 +82,9 @@ struct StageArgs {
     int kernel_choice;     // whole-mesh float 2D stages: 0 automatic, 1 tile kernel, 2 persistent kernel
     int tile_row0;         // 2D: first tile row of the launch
     int tile_rows;         // 2D: tile rows of the launch (0: through the last row of the mesh)
-    int pdl;               // 1: the launch may begin while the kernel before it in its stream drains
-                           // (programmatic dependent launch; sequences of whole-mesh stages)
+    int pdl;               // the launch may begin while the kernel before it in its stream drains
+                           // (programmatic dependent launch; sequences of whole-mesh stages):
+                           // kPdlDirect if launched one by one, kPdlCaptured into a graph, 0 not
     int wait_limit;        // polls of a bounded TMA wait: 0 the default limit, < 0 none (the
                            // wait gives up at once; diagnostic)
     // prescribed-state sides (2D Euler, DGW_BC_STATE): the stage's time is *t_dev + t_off

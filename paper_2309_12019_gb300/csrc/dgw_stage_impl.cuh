@@ -201,13 +201,18 @@ __device__ __forceinline__ double sensor_ratio(double qd, double beta0, double W
 
 constexpr double kPi = 3.14159265358979323846;
 
-// Start of a kernel that may be launched while the one before it drains: lets the next launch
-// begin as soon as all CTAs of this one run, then waits until everything before is complete and
-// visible.  Without the launch attribute both are no-ops.
+// Start of a kernel that may be launched while the one before it drains: waits until everything
+// before is complete and visible, then lets the next launch begin as soon as all CTAs of this one
+// run.  In this order two launches of a sequence are resident at most; the other way round the CTAs of
+// the launch after next fill the SMs too, unevenly (2D Euler 96^2 Q2 FP32 replayed, 9.6 -> 7.6 us a
+// stage).  EARLY: the other way round, for kernels whose launches are bound by the host.
+// Without the launch attribute both are no-ops.
+template <bool EARLY = false>
 __device__ __forceinline__ void pdl_begin()
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Products and sums rounded one way in every kernel that inlines them (intrinsics are not
@@ -1584,26 +1589,6 @@ __global__ void __launch_bounds__(TX * kPThreadRows, 1) stage_kernel_p(const __g
 }
 #endif
 
-// Launches a kernel, with pdl as a programmatic dependent launch: it may start while the kernel
-// before it in the stream drains.  Every kernel launched so begins with pdl_begin, so nothing of
-// it runs early but the launch itself and the first CTAs.  Per stage: Sod train 95.5 -> 91.8 us,
-// triple point 65.6 -> 62.7, KPP 1024^2 100.9 -> 98.8, 42^2 cells of 2D Euler 8.5 -> 6.8.
-template <class... Args>
-static cudaError_t launch_k(void (*fn)(Args...), dim3 grid, dim3 block, size_t smem, bool pdl, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, fn, args...);
-}
-
 // Current device, for per-device caches of kernel attributes (0 if it cannot be read or
 // lies beyond the caches' 64 entries).
 static int cur_device()
@@ -1614,7 +1599,7 @@ static int cur_device()
 }
 
 // SMs of the current device (0 if it cannot be read)
-[[maybe_unused]] static int sm_count()
+static int sm_count()
 {
     static int nsm[64] = {0};
     int dev = 0;
@@ -1622,6 +1607,53 @@ static int cur_device()
     if (nsm[dev] == 0 && cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         nsm[dev] = 0;
     return nsm[dev];
+}
+
+constexpr size_t kMaxSmemSm = 228 * 1024, kMaxSmemCta = 227 * 1024;   // 1 KB of each CTA's is reserved
+
+// Launches FN, with pdl as a programmatic dependent launch: it may start while the kernel before it
+// drains.  Every kernel launched so begins with pdl_begin, so nothing of it runs early but the launch
+// itself and the first CTAs.  It hides 2 us between launches made one by one (kPdlDirect), 0.1 to
+// 0.3 us between those of a graph (kPdlCaptured).  But CTAs that come early go to whichever SMs have
+// room beside the kernel before: if an SM holds more of them (occ) than its share, some SMs get occ and
+// others too few, and a kernel that is bound by throughput takes up to occ / ceil(CTAs / SMs) times as
+// long.  KPP 256^2 Q1 FP64, us a stage: 155 without, 215 with; 2D Euler 128^2 Q1 FP64 83 and 177.  So
+// where a mesh's CTAs leave an SM room for more than its share,
+//   PAD (kernels whose shared memory is dynamic): more of it is asked for, so that an SM holds its share
+//     only: KPP 146, 2D Euler 74;
+//   else no early start beyond one CTA per SM (beyond half of that in a graph, where little is lost):
+//     1D Burgers 32768 cells Q2 FP64, 40 without this rule, 16 with it;
+//   but float launches made one by one always start early: their stages of such sizes are mostly
+//     latency (Burgers 333 x 217 Q1: 8.0 with the other order of pdl_begin, 8.2 without an early
+//     start, 6.9 padded, 6.3 so).
+template <auto FN, bool PAD = false, class... Args>
+static cudaError_t launch_k(dim3 grid, dim3 block, size_t smem, int pdl, cudaStream_t st, Args... args)
+{
+    if (pdl != 0 && (PAD || !(pdl == kPdlDirect && kF32))) {
+        static int known[64] = {0};      // CTAs that an SM holds
+        int occ = __atomic_load_n(&known[cur_device()], __ATOMIC_RELAXED);
+        if (occ == 0) {
+            const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, FN, block.x * block.y, smem);
+            if (e != cudaSuccess) return e;
+            __atomic_store_n(&known[cur_device()], occ, __ATOMIC_RELAXED);
+        }
+        const long long n = (long long)grid.x * grid.y, nsm = sm_count();
+        if (n <= (occ - 1) * nsm) {
+            if constexpr (PAD) smem = std::max(smem, (size_t)(kMaxSmemSm / ((n + nsm - 1) / nsm) - 1024) / 128 * 128);
+            else if ((pdl == kPdlDirect ? n : 2 * n) > nsm) pdl = 0;
+        }
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl != 0 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, FN, args...);
 }
 
 static KParams make_params(const StageArgs& s)
@@ -1931,9 +1963,9 @@ static cudaError_t launch_vjp_p(const StageArgs& s, int flux, const void* lam, v
     const KParams a = make_params(s);
     const unsigned blocks = (unsigned)((s.E + 127) / 128);
     if (flux == FLUX_ADVECT)
-        return launch_k(vjp_kernel<P, FLUX_ADVECT>, blocks, 128, 0, s.pdl != 0, st, a, (const Real*)lam, (Real*)wself, (Real*)wnb);
+        return launch_k<vjp_kernel<P, FLUX_ADVECT>>(blocks, 128, 0, s.pdl, st, a, (const Real*)lam, (Real*)wself, (Real*)wnb);
     if (flux == FLUX_BURGERS)
-        return launch_k(vjp_kernel<P, FLUX_BURGERS>, blocks, 128, 0, s.pdl != 0, st, a, (const Real*)lam, (Real*)wself, (Real*)wnb);
+        return launch_k<vjp_kernel<P, FLUX_BURGERS>>(blocks, 128, 0, s.pdl, st, a, (const Real*)lam, (Real*)wself, (Real*)wnb);
     return cudaErrorInvalidValue;
 }
 
@@ -1956,9 +1988,9 @@ static cudaError_t launch_gather(const GatherArgs& g, int p, cudaStream_t st)
     const Real* x2 = (const Real*)g.x[2];
     const Real c0 = (Real)g.coef[0], c1 = (Real)g.coef[1], c2 = (Real)g.coef[2], cv = (Real)g.cvjp;
     switch (p) {
-    case 1: return launch_k(gather_kernel<1>, blocks, 128, 0, g.pdl != 0, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
-    case 2: return launch_k(gather_kernel<2>, blocks, 128, 0, g.pdl != 0, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
-    case 3: return launch_k(gather_kernel<3>, blocks, 128, 0, g.pdl != 0, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
+    case 1: return launch_k<gather_kernel<1>>(blocks, 128, 0, g.pdl, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
+    case 2: return launch_k<gather_kernel<2>>(blocks, 128, 0, g.pdl, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
+    case 3: return launch_k<gather_kernel<3>>(blocks, 128, 0, g.pdl, st, g.E, g.nx, g.ny, (const Real*)g.wself, (const Real*)g.wnb, x0, x1, x2, c0, c1, c2, cv, (Real*)g.out);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -2027,7 +2059,7 @@ static bool persistent_pays(int nx, int ny)
 }
 
 template <int P, int FLUX>
-static cudaError_t launch_persistent(const KParams& a, bool pdl, cudaStream_t st)
+static cudaError_t launch_persistent(const KParams& a, int pdl, cudaStream_t st)
 {
     constexpr size_t smem = p_smem_bytes<P>();
     static_assert(smem <= 227 * 1024, "persistent tile exceeds the shared memory of an SM");
@@ -2041,12 +2073,12 @@ static cudaError_t launch_persistent(const KParams& a, bool pdl, cudaStream_t st
     const int nsm = sm_count();
     const int ntiles = ((a.nx + TX - 1) / TX) * ((a.ny + kPRows - 1) / kPRows);
     if (ntiles == 0) return cudaSuccess;
-    return launch_k(stage_kernel_p<P, FLUX>, ntiles < nsm ? ntiles : nsm, TX * kPThreadRows, smem, pdl, st, a);
+    return launch_k<stage_kernel_p<P, FLUX>>(ntiles < nsm ? ntiles : nsm, TX * kPThreadRows, smem, pdl, st, a);
 }
 #endif
 
 template <int P, int FLUX, int MODE, bool DENSE>
-static cudaError_t launch_tile(const KParams& a, dim3 grid, size_t smem, bool pdl, cudaStream_t st)
+static cudaError_t launch_tile(const KParams& a, dim3 grid, size_t smem, int pdl, cudaStream_t st)
 {
     // once per instantiation and device: opt in to more than 48 KB of dynamic shared
     // memory where needed, and prefer the largest shared-memory carveout (several tiles per SM)
@@ -2055,13 +2087,13 @@ static cudaError_t launch_tile(const KParams& a, dim3 grid, size_t smem, bool pd
     if (!opted[dev]) {
         const void* fn = (const void*)stage_kernel<P, FLUX, MODE, DENSE>;
         cudaError_t e = cudaSuccess;
-        if (smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemCta);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         opted[dev] = true;
     }
-    return launch_k(stage_kernel<P, FLUX, MODE, DENSE>, grid, NTS, smem, pdl, st, a);
+    return launch_k<stage_kernel<P, FLUX, MODE, DENSE>, DIM == 2 && !kF32>(grid, NTS, smem, pdl, st, a);
 }
 
 template <int P, int FLUX>
@@ -2079,15 +2111,15 @@ static cudaError_t launch_pf(const StageArgs& s, int mode, cudaStream_t st)
     if constexpr (kF32) {
         if (mode == 0 && s.tmap_p && s.tile_row0 == 0 && s.tile_rows == 0 && (!a.has_un || a.use_p_un) &&
             (s.kernel_choice == 2 || persistent_pays<P, FLUX>(s.nx, s.ny)))
-            return launch_persistent<P, FLUX>(a, s.pdl != 0, st);
+            return launch_persistent<P, FLUX>(a, s.pdl, st);
     }
     if constexpr (stage_blocks<P>(true) != stage_blocks<P>(false)) {
         if (mode == 0 && (long long)grid.x * grid.y > (long long)stage_blocks<P>(false) * sm_count())
-            return launch_tile<P, FLUX, 0, true>(a, grid, smem, s.pdl != 0, st);
+            return launch_tile<P, FLUX, 0, true>(a, grid, smem, s.pdl, st);
     }
 #endif
-    return mode == 0 ? launch_tile<P, FLUX, 0, false>(a, grid, smem, s.pdl != 0, st)
-                     : launch_tile<P, FLUX, 1, false>(a, grid, smem, s.pdl != 0, st);
+    return mode == 0 ? launch_tile<P, FLUX, 0, false>(a, grid, smem, s.pdl, st)
+                     : launch_tile<P, FLUX, 1, false>(a, grid, smem, s.pdl, st);
 }
 
 template <int P>
