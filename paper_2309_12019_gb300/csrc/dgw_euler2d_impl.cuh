@@ -4,11 +4,11 @@
 //
 // State U = (rho, rho vx, rho vy, rho E), p = (gamma - 1)(rho E - rho |v|^2 / 2); mode
 // k = i + (p+1) j of component comp of cell e at row comp K + k, K = (p+1)^2.
-// One CTA of 32 x EY threads owns a tile of as many cells, one per thread:
+// One CTA of EX x EY = 32 x 4 threads owns a tile of as many cells, one per thread:
 //   0. the tile's coefficients and a one-cell face halo (all four components) are
 //      staged in shared memory by asynchronous copies of words; halo cells beyond a periodic side
-//      are its images, beyond a wall or an outflow side they are absent; in float the
-//      Un coefficients of the tile start to arrive by cp.async
+//      are its images, beyond a wall or an outflow side they are absent; the tile's Un is
+//      asked for into L2
 //   1. per cell: the sensor of Sec. 4 on the density, the volume term at the (p+2)^2
 //      Gauss points by sum factorisation, lambda_e over those points
 //   2. every face of the tile once: both traces at the p+2 Gauss points, the ghost
@@ -20,22 +20,27 @@
 // Constants are folded as in the scalar kernel:
 //   L_k = (2/h) minv(i) minv(j) [acc_k - gamma lambda / p (K_ref c)_k].
 
-// Tile heights: 8 rows (256 threads, two CTAs per SM) in float up to p = 2, else 4.  The kernel is
-// bound by instruction issue and by the latency of its dependent operations, so it wants warps:
-// with the tile's Un in shared memory 3 CTAs of 4 rows fitted (12 warps, issue active 59 %); Un
-// is now prefetched into L2 and read into registers after the faces, which makes room for 16
-// warps, and the taller tile has fewer halo cells and faces per cell.  Kelvin-Helmholtz 2048^2, p = 2,
-// FP32: 746 -> 680 us a stage; triple point 896 x 384: 69 -> 66 us.  The tile's coefficients arrive by
-// cp.async, all in flight at once; loads into registers stalled the warps for a third of the time
-// (675 -> 629 us and 62.7 -> 56.7 us).
+// Tiles of 4 rows, 128 threads.  The kernel is bound by instruction issue and by the latency of its
+// dependent operations, so it wants warps, and CTAs that are at different phases: in float five
+// CTAs per SM at p = 1 (79 registers), four at p = 2 (128), two at p = 3 (230).  Un in shared memory
+// would leave room for three at p = 2 (12 warps, issue active 59 %), so it is prefetched into L2 and
+// read into registers after the faces.  Tiles of 8 rows have fewer halo cells and faces per cell but
+// half the CTAs, whose warps meet at the same barriers.  us a stage, FP32, 8 rows with two CTAs per
+// SM / 4 rows:
+//   p = 1:  64^2 5.9 / 4.9,  128^2 6.9 / 5.1,  224^2 7.7 / 7.1,  256^2 7.7 / 8.1,  512^2 23.0 / 21.0,  1024^2 83.6 / 74.8
+//   p = 2:  64^2 9.7 / 7.6,  128^2 12.0 / 7.8,  224^2 13.7 / 12.1,  512^2 43.1 / 41.8,  1024^2 157 / 148;
+//           Kelvin-Helmholtz 2048^2 613 / 582, triple point 57.3 / 54.5
+// At p = 3 Un in shared memory instead of 28 more registers is slower too (1024^2 329 late, 368 shared).
+// The tile's coefficients arrive by cp.async, all in flight at once; loads into registers stalled the
+// warps for a third of the time (Kelvin-Helmholtz 675 -> 629 us).
 using R2 = std::conditional_t<kF32, float2, double2>;   // a pair of state components
 constexpr int EX = kTileX2, EHX = EX + 2;               // tile columns, staged columns
-template <int P> constexpr int euler2_rows() { return kF32 && P <= 2 ? 8 : kTileY2; }
-template <int P> constexpr int euler2_blocks() { return 2; }
+constexpr int EY = kTileY2;
+template <int P> constexpr int euler2_blocks() { return !kF32 || P == 3 ? 2 : (P == 2 ? 4 : 5); }
 
 template <int P>
 struct Euler2Smem {
-    static constexpr int N1 = P + 1, K = N1 * N1, EY = euler2_rows<P>(), EHY = EY + 2;
+    static constexpr int N1 = P + 1, K = N1 * N1, EHY = EY + 2;
     // the four components as two pairs (rho, rho vx), (rho vy, rho E), each pair one
     // 8-byte (float) or 16-byte (double) word, so that a pair is one shared load or store
     R2 u[2][K][EHY][EHX];           // coefficients; tile cell (lx, ly) at [ly + 1][lx + 1]
@@ -157,10 +162,10 @@ __device__ __forceinline__ Real sensor_2d(const KParams& A, const Tab<P>& T, con
 
 // MODE 0: stage / residual; MODE 1: sensor only (writes gamma_out).
 template <int P, int MODE>
-__global__ void __launch_bounds__(EX * euler2_rows<P>(), euler2_blocks<P>()) euler2d_kernel(const __grid_constant__ KParams A)
+__global__ void __launch_bounds__(EX * EY, euler2_blocks<P>()) euler2d_kernel(const __grid_constant__ KParams A)
 {
     constexpr int N1 = P + 1, NQ = P + 2, K = N1 * N1;
-    constexpr int EY = euler2_rows<P>(), ENT = EX * EY, EHY = EY + 2;
+    constexpr int ENT = EX * EY, EHY = EY + 2;
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_e2[];
     Euler2Smem<P>& S = *reinterpret_cast<Euler2Smem<P>*>(smem_e2);
@@ -486,7 +491,6 @@ static cudaError_t launch_euler2d_p(const StageArgs& s, int mode, cudaStream_t s
     KParams a = make_params(s);
     // (states that L2 holds are not asked for ahead: the triple point's 50 MB gain nothing)
     a.round_tiles = kF32 && (double)s.E * 4 * Tab<P>::K * sizeof(Real) > 64e6 ? euler2_blocks<P>() * sm_count() : 0;
-    constexpr int EY = euler2_rows<P>();
     dim3 grid((s.nx + EX - 1) / EX, (s.ny + EY - 1) / EY);
     if (grid.x == 0 || grid.y == 0) return cudaSuccess;
     const size_t smem = sizeof(Euler2Smem<P>);
