@@ -67,7 +67,9 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
     const int me = (has[0] ? 1 : 0) + (has[1] ? 1 : 0);
     const Real beta0 = qform<P>(T, c);
     const Real d0 = A.eps_w + beta0;
-    const Real w0 = div_w(Real(1) - Real(me) * A.w_nbr, d0 * d0);
+    Real own = Real(1) - Real(me) * A.w_nbr, nbr = A.w_nbr;     // numerators of the weights
+    if (TILE) scale_weights(d0, own, nbr);
+    const Real w0 = div_w(own, d0 * d0);
     Real wsum = w0;
     Real wnb[2] = {Real(0), Real(0)};
     Real dacc[N1];
@@ -88,7 +90,7 @@ __device__ __forceinline__ Real sensor_1d(const KParams& A, const Tab<P>& T, con
             cl[k] = s;
         }
         const Real dl = A.eps_w + qform<P>(T, cl);
-        const Real wl = div_w(A.w_nbr, dl * dl);
+        const Real wl = div_w(nbr, dl * dl);
         wsum += wl;
         wnb[f] = wl;
 #pragma unroll

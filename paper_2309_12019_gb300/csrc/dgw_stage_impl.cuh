@@ -173,16 +173,34 @@ __device__ __forceinline__ float max_pos(float a, float b) { return fmaxf(a, b);
 __device__ __forceinline__ double max_pos(double a, double b) { return less_pos(a, b) ? b : a; }
 
 // a / b for the sensor weights: the hardware reciprocal in float (at most 2 ulp; the
-// divisors here lie in [1e-12, 1e30]), the correctly rounded quotient in double.
+// divisors here lie in [1e-12, 1e30]); in double the product with the rounded reciprocal (two
+// roundings: the sensor's error against 64 bits is the same with the quotient, within 1 %).
 __device__ __forceinline__ float div_w(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double div_w(double a, double b) { return a * __drcp_rn(b); }
 
-// gamma of Eq. (sensor / gensensor) before the exponent q, min(1, r) with r = ||D|| / (W ||U||)
-// through the squares qd = ||D||^2, beta0 = ||U||^2 and W^2: one reciprocal square root in place
-// of two square roots and two divisions (double; the products stay in range while qd W^2 beta0
-// does, else the roots are taken one by one).  rr receives r (1 if not below 1).  With the integer
-// comparisons: rotation at 256^2 Q2, 149 -> 142 us a stage (tiles of 2 rows in place of 4, which
-// load the SMs more evenly there, 149).
+// Numerators of a cell's sensor weights, the cell's own and its neighbours', for states far above one
+// in double: the weights go with U^-4 and the squares that sensor_ratio takes with U^-8, which underflow
+// from U = 1e40 on, so both are multiplied by a power of two near U (only their ratios matter, and
+// the power of two changes no bit of these).  d0 = eps_w + ||U||^2.
+__device__ __forceinline__ void scale_weights(double d0, double& own, double& nbr)
+{
+    const int h = __double2hiint(d0);
+    if (h > (1023 + 64) << 20) {
+        const double s = __hiloint2double((((h >> 20) - 1023) / 2 + 1023) << 20, 0);
+        own *= s;
+        nbr *= s;
+    }
+}
+
+__device__ __forceinline__ void scale_weights(float, float&, float&) {}    // (float divides D by W first)
+
+// gamma of Eq. (sensor / gensensor) before the exponent q, min(1, r) with r = ||D|| / (W ||U||),
+// D = sum_l w_l (c - c_l), through the squares qd = ||D||^2, beta0 = ||U||^2 and W^2: one reciprocal
+// square root in place of two square roots and two divisions (double; the products stay in range
+// while qd W^2 beta0 does, else the roots are taken one by one).  rr receives r (1 if not below 1).
+// The error against 64 bits is that of the roots and quotients, 2.2 to 2.9 units of 2^-53 rms on
+// random states.  With the integer comparisons: rotation at 256^2 Q2, 149 -> 142 us a stage (tiles of 2
+// rows in place of 4, which load the SMs more evenly there, 149).
 __device__ __forceinline__ double sensor_ratio(double qd, double beta0, double W, double eps_s, double* rr)
 {
     const double W2 = W * W, den = W2 * beta0, pr = qd * den;
@@ -852,6 +870,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
     V gamma = vbc<V>((MODE == 0 && A.stab == STAB_LO) ? Real(1) : Real(0));
     if ((MODE == 1 || A.stab >= STAB_WENO) && any_in) {
         bool has[2 * DIM][L];   // face neighbour f of lane l's cell exists
+        Real nbr = A.w_nbr;     // numerator of the neighbours' weights
         V wsum;
         V wnb[2 * DIM];         // unnormalised neighbour weights (zero where missing)
         const V beta0 = qform<P>(T, c);
@@ -866,7 +885,9 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
                 has[f][l] = (f < 2) ? (wrap_x(A, nx_) >= 0) : (wrap_y(A, ny_) >= 0);
                 me += has[f][l] ? 1 : 0;
             }
-            lane(wsum, l) = div_w(Real(1) - Real(me) * A.w_nbr, lane(d0, l) * lane(d0, l));
+            Real own = Real(1) - Real(me) * A.w_nbr;
+            if constexpr (!kF32) scale_weights(d0, own, nbr);
+            lane(wsum, l) = div_w(own, lane(d0, l) * lane(d0, l));
         }
         const V w0 = wsum;      // unnormalised weight of the cell's own candidate
         V dacc[K];
@@ -907,7 +928,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             V wl;
 #pragma unroll
             for (int l = 0; l < L; ++l)
-                lane(wl, l) = has[f][l] ? div_w(A.w_nbr, lane(dl, l) * lane(dl, l)) : Real(0);
+                lane(wl, l) = has[f][l] ? div_w(nbr, lane(dl, l) * lane(dl, l)) : Real(0);
             wsum = vadd(wsum, wl);
             wnb[f] = wl;
 #pragma unroll
