@@ -797,10 +797,7 @@ extern "C" dgw_status dgw_rk_step_host(dgw_ctx* c, const void* U_in, void* U_out
 // by sum factorisation, two sample rows (+-g_b) at a time, each sample read once.  On the
 // symmetric Gauss nodes P_i(-g) = +-P_i(g), so sums over +-pairs halve the multiplications.
 // Double states and 1D: the sums in double, 288 operations a cell at 8 x 8 samples and p = 3; the
-// FP64 pipe (2 lanes per SM) bounds them, not memory.  Float states in 2D: project_split_kernel.
-// 1024^2 cells, p = 3, 8 x 8 samples, with the mass that follows: the direct double loop over modes
-// (2688 operations, every sample read K times) took 4.53 ms, this in double 0.73 ms, split
-// 0.20 ms (the 604 MB it moves would take 0.09 ms).
+// FP64 pipe (2 lanes per SM) bounds them, not memory.  Float states in 2D: project_fixed_kernel.
 struct ProjArgs {
     const double* f;
     void* U;
@@ -809,7 +806,7 @@ struct ProjArgs {
     int vec;                        // sample rows start on 16-byte boundaries
     double WB[8][kMaxN1];           // w_q P_i(g_q)
     double minv[kMaxN1];
-    float sh[8][kMaxN1], sl[8][kMaxN1];   // minv_i w_q P_i(g_q) = sh + sl to 48 bits
+    int mh[8][kMaxN1], ml[8][kMaxN1];   // minv_i w_q P_i(g_q) 2^60 = mh 2^31 + ml
 };
 
 // out[i] = sum_q WB[q][i] f[q] on symmetric nodes
@@ -905,134 +902,180 @@ __global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ Pr
     if (e < a.E) project_cell<DIM, N1, NQ>(a, e);
 }
 
-// Two lanes of unevaluated sums hi + lo (|lo| at most a few 2^-23 |hi|): the double-float
-// arithmetic of Dekker, "A floating-point technique for extending the available precision" (1971),
-// with the product's error from an FMA.  Every value carries 46 bits or more, so the float that
-// hi + lo is rounded to at the end is that of the sums in double but for values within 2^-20 of a
-// rounding boundary: of 4 million modes of the 1024^2 Q3 KPP data a few differ by one rounding, and
-// the error against 64 bits is the same 2.5e-8.
-struct Split2 {
-    float2 hi, lo;
-};
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-// s + *err = a + b exactly (Knuth's two-sum)
-__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2* err)
+// Float states in 2D: the sums of project_cell in 64-bit fixed point, on integer multipliers that are
+// several times as wide as the FP64 pipe.  Per cell the samples become integers of 59 bits (the unit from
+// the largest exponent), the centre sample is taken off them, exactly, and the differences d are
+// shifted up to 60 bits, so that all errors are relative to the cell's variation: fewer than
+// five roundings of 2^-57 max |d| in a mode, where the double sums round by 2^-53 of the samples or of
+// their differences.  The stored modes' error against 64 bits is the double sums' or less in every mode,
+// on smooth data whose high modes cancel too (2 + sin cos on 64^2 to 1024^2 cells, p = 3, Kelvin-Helmholtz,
+// KPP, cones, noise).  (The centre sample meets only the mean: rules of two points or more annihilate
+// P_1 to P_3.)  Products take two limbs of 31 bits each: with x = xh 2^31 + xl and the weight M 2^60 =
+// mh 2^31 + ml, M x = 4 sum mh xh + 2^-29 sum (mh xl + ml xh) but for one unit; |M| < 2, sum |M| < 2.7 and
+// |x| < 2^61 keep every sum below 2^63.  Cells with samples that are not finite, or largest ones
+// outside [2^-60, 2^100), take the sums in double.
+// The samples arrive through shared memory, whole lines at a time; 65 words a cell keep the lanes
+// that read one cell each on banks of their own.  1024^2 cells, p = 3, 8 x 8 samples, with the mass that
+// follows: every sample read K times in double 4.53 ms, project_cell in double 0.73 ms, this 0.29 ms
+// (604 MB would take 0.09 ms; the pipe of the 64-bit multiply-adds, 576 a cell, is 73 % busy).
+constexpr int kProjFixedThreads = 64;
+__device__ __forceinline__ void proj_limbs(long long x, int& h, int& l)
 {
-    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
-    *err = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
-    return s;
+    h = (int)(x >> 31);
+    l = (int)((unsigned)x & 0x7fffffffu);
 }
-__device__ __forceinline__ Split2 split_add(Split2 a, Split2 b)
+// A 2^62 + B 2^31 += (M x) 2^60
+__device__ __forceinline__ void proj_mad(int mh, int ml, int h, int l, long long& A, long long& B)
 {
-    Split2 r;
-    float2 e;
-    r.hi = two_sum(a.hi, b.hi, &e);
-    r.lo = __fadd2_rn(__fadd2_rn(a.lo, b.lo), e);
-    return r;
+    A += (long long)mh * h;
+    B += (long long)mh * l;
+    B += (long long)ml * h;
 }
-__device__ __forceinline__ Split2 split_neg(Split2 a)
+// v as an integer multiple (rounded down in magnitude) of 2^(X - 1023 - 58), X the largest biased
+// exponent of the cell
+__device__ __forceinline__ long long proj_fixed(double v, int X)
 {
-    return {make_float2(-a.hi.x, -a.hi.y), make_float2(-a.lo.x, -a.lo.y)};
-}
-// acc + (wh + wl) x
-__device__ __forceinline__ Split2 split_fma(float2 wh, float2 wl, Split2 x, Split2 acc)
-{
-    const float2 p = __fmul2_rn(wh, x.hi);
-    float2 e = __ffma2_rn(wh, x.hi, make_float2(-p.x, -p.y)), t;
-    e = __ffma2_rn(wh, x.lo, e);
-    e = __ffma2_rn(wl, x.hi, e);
-    Split2 r;
-    r.hi = two_sum(acc.hi, p, &t);
-    r.lo = __fadd2_rn(acc.lo, __fadd2_rn(t, e));
-    return r;
-}
-// v as hi + lo, from its bits (a conversion would occupy the FP64 pipe): the leading 24 and the
-// next 23 bits of the significand.  Zero is exact; other values outside [2^-60, 2^96) set *bad.
-__device__ __forceinline__ void split_double(double v, float* hi, float* lo, bool* bad)
-{
-    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
-    const bool ok = (h & 0x7fffffffu) - 0x3c300000u < 0x45f00000u - 0x3c300000u;
-    *bad = *bad || (!ok && ((h & 0x7fffffffu) | l) != 0u);
-    // bits 30 .. 23 of the shifted word are the exponent mod 256, 1023 + x; float wants 127 + x
-    const unsigned bits = ((__funnelshift_l(l, h, 3) ^ 0x40000000u) & 0x7fffffffu) | (h & 0x80000000u);
-    const unsigned base = (bits & 0xff800000u) - (23u << 23);
-    const float d = __uint_as_float(base | ((l >> 6) & 0x7fffffu)) - __uint_as_float(base);
-    *hi = ok ? __uint_as_float(bits) : 0.f;
-    *lo = ok ? d : 0.f;
+    const int h = __double2hiint(v);
+    const unsigned long long m = ((unsigned long long)((h & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+    const long long q = (long long)((m << 6) >> min(X - ((h >> 20) & 0x7ff), 63));
+    return h < 0 ? -q : q;
 }
 
-// Float states in 2D: the sums of project_cell on the packed FP32 pipe, which is 64 times as wide as
-// the FP64 one, in double-float arithmetic.  The lanes of a pair are the rows +-g_b while the
-// points of a row are summed, then the even and the odd mode j.  Cells with samples that the split
-// cannot hold (tiny, huge, not finite) take the sums in double.
 template <int N1, int NQ>
-__global__ void __launch_bounds__(128) project_split_kernel(const __grid_constant__ ProjArgs a)
+__global__ void __launch_bounds__(kProjFixedThreads) project_fixed_kernel(const __grid_constant__ ProjArgs a)
 {
-    constexpr int NP = NQ / 2, NR = (NQ + 1) / 2, NJ = (N1 + 1) / 2;
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int NPT = NQ * NQ, ST = NPT | 1, NP = NQ / 2, NT = kProjFixedThreads;
+    __shared__ double sm[NT * ST];
+    const int64_t e0 = (int64_t)blockIdx.x * NT, e = e0 + threadIdx.x;
+    const int n = (int)(a.E - e0 < NT ? a.E - e0 : NT);
+    const double* src = a.f + e0 * NPT;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n * NPT; i += NT) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sm[i / NPT * ST + i % NPT]);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(dst), "l"(src + i) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
     if (e >= a.E) return;
-    const double* f = a.f + e * (NQ * NQ);
-    const float2 zero = make_float2(0.f, 0.f);
-    bool bad = false;
-    Split2 c[N1][NJ];
+    double* const f = sm + threadIdx.x * ST;
+    long long* const d = reinterpret_cast<long long*>(f);
+    float* const U = static_cast<float*>(a.U) + e;
+
+    const double f0 = f[NQ / 2 * NQ + NQ / 2];
+    const int h0 = __double2hiint(f0);
+    int top = 0, diff = 0;               // largest |f|; bits in which the upper words differ
+#pragma unroll
+    for (int i = 0; i < NPT; ++i) {
+        const int h = __double2hiint(f[i]);
+        top = max(top, h & 0x7fffffff);
+        diff |= h ^ h0;
+    }
+    const int X = top >> 20;
+    if (X != 0 && (X < 1023 - 60 || X >= 1023 + 100)) {
+        project_cell<2, N1, NQ>(a, e);
+        return;
+    }
+    int bits = 0;                        // set bits of the upper words of |d|
+    int neg = 0;                         // d is taken of -f
+    if ((diff & 0xfff00000) == 0) {
+        // one sign and exponent (or all zero): the difference of the bits is that of the significands
+        const long long b0 = __double_as_longlong(f0);
+        neg = h0 < 0;
+#pragma unroll 16
+        for (int i = 0; i < NPT; ++i) {
+            const long long q = (d[i] - b0) * 64;
+            const int h = (int)(q >> 32);
+            bits |= h ^ (h >> 31);
+            d[i] = q;
+        }
+    } else {
+        const long long q0 = proj_fixed(f0, X);
+#pragma unroll 8
+        for (int i = 0; i < NPT; ++i) {
+            const long long q = proj_fixed(f[i], X) - q0;
+            const int h = (int)(q >> 32);
+            bits |= h ^ (h >> 31);
+            d[i] = q;
+        }
+    }
+    unsigned long long mask = (unsigned long long)(unsigned)bits << 32;
+    if (bits == 0)                       // (all below 2^-27 of the largest sample)
+        for (int i = 0; i < NPT; ++i) mask |= (unsigned long long)(d[i] ^ (d[i] >> 63));
+    if (mask == 0 || X == 0) {           // a constant, or nothing but zeros and numbers below the normal ones
+#pragma unroll
+        for (int k = 0; k < N1 * N1; ++k) U[k * a.E] = k == 0 ? (float)f0 : 0.f;
+        return;
+    }
+    const int up = __clzll((long long)mask) - 4;
+    auto shl = [up](long long v) { return (long long)((unsigned long long)v << up); };
+
+    long long A[N1][N1], B[N1][N1];
 #pragma unroll
     for (int i = 0; i < N1; ++i)
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) c[i][j] = {zero, zero};
-#pragma unroll 1
-    for (int m = 0; m < NR; ++m) {
-        // rows m (lane x) and NQ - 1 - m (lane y); the centre row of an odd rule alone
-        const int mp = NQ - 1 - m;
-        double rm[NQ], rp[NQ];
-        proj_row<NQ>(f, m, a.vec, rm);
-        proj_row<NQ>(f, mp, a.vec, rp);
-        Split2 x[NQ];
+        for (int j = 0; j < N1; ++j) A[i][j] = B[i][j] = 0;
+    // quarters of the x-sums of row b
+    auto row = [&](int b, long long (&r)[N1]) {
+        long long ra[N1], rb[N1];
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            split_double(rm[q], &x[q].hi.x, &x[q].lo.x, &bad);
-            split_double(rp[q], &x[q].hi.y, &x[q].lo.y, &bad);
-            if ((NQ & 1) != 0 && m == mp) x[q].hi.x = x[q].lo.x = 0.f;
-        }
-        Split2 r[N1];
-#pragma unroll
-        for (int i = 0; i < N1; ++i) r[i] = {zero, zero};
+        for (int i = 0; i < N1; ++i) ra[i] = rb[i] = 0;
         if constexpr ((NQ & 1) != 0) {
+            int h, l;
+            proj_limbs(shl(d[b * NQ + NP]), h, l);
 #pragma unroll
-            for (int i = 0; i < N1; i += 2)
-                r[i] = split_fma(make_float2(a.sh[NP][i], a.sh[NP][i]), make_float2(a.sl[NP][i], a.sl[NP][i]), x[NP], r[i]);
+            for (int i = 0; i < N1; i += 2) proj_mad(a.mh[NP][i], a.ml[NP][i], h, l, ra[i], rb[i]);
         }
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             const int qp = NQ - 1 - q;
-            const Split2 S = split_add(x[qp], x[q]), D = split_add(x[qp], split_neg(x[q]));
+            const long long x = shl(d[b * NQ + qp]), y = shl(d[b * NQ + q]);
+            int sh, sl, dh, dl;
+            proj_limbs(x + y, sh, sl);
+            proj_limbs(x - y, dh, dl);
 #pragma unroll
-            for (int i = 0; i < N1; ++i)
-                r[i] = split_fma(make_float2(a.sh[qp][i], a.sh[qp][i]), make_float2(a.sl[qp][i], a.sl[qp][i]), (i & 1) ? D : S, r[i]);
+            for (int i = 0; i < N1; ++i) proj_mad(a.mh[qp][i], a.ml[qp][i], (i & 1) ? dh : sh, (i & 1) ? dl : sl, ra[i], rb[i]);
         }
+#pragma unroll
+        for (int i = 0; i < N1; ++i) r[i] = ra[i] + ((rb[i] + (1ll << 30)) >> 31);
+    };
+    if constexpr ((NQ & 1) != 0) {
+        long long r[N1];
+        row(NP, r);
 #pragma unroll
         for (int i = 0; i < N1; ++i) {
-            // (r+ + r-, r+ - r-): what the even and the odd modes j take
-            const Split2 p = {make_float2(r[i].hi.y, r[i].hi.y), make_float2(r[i].lo.y, r[i].lo.y)};
-            const Split2 n = {make_float2(r[i].hi.x, -r[i].hi.x), make_float2(r[i].lo.x, -r[i].lo.x)};
-            const Split2 sd = split_add(p, n);
+            int h, l;
+            proj_limbs(r[i], h, l);
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int j1 = 2 * j + 1 < N1 ? 2 * j + 1 : 2 * j;
-                c[i][j] = split_fma(make_float2(a.sh[mp][2 * j], a.sh[mp][j1]), make_float2(a.sl[mp][2 * j], a.sl[mp][j1]), sd, c[i][j]);
-            }
+            for (int j = 0; j < N1; j += 2) proj_mad(a.mh[NP][j], a.ml[NP][j], h, l, A[i][j], B[i][j]);
         }
     }
-    if (bad) {
-        project_cell<2, N1, NQ>(a, e);
-        return;
+#pragma unroll 1
+    for (int m = 0; m < NP; ++m) {
+        const int mp = NQ - 1 - m;
+        long long rm[N1], rp[N1];
+        row(m, rm);
+        row(mp, rp);
+#pragma unroll
+        for (int i = 0; i < N1; ++i) {
+            int sh, sl, dh, dl;
+            proj_limbs(rp[i] + rm[i], sh, sl);
+            proj_limbs(rp[i] - rm[i], dh, dl);
+#pragma unroll
+            for (int j = 0; j < N1; ++j) proj_mad(a.mh[mp][j], a.ml[mp][j], (j & 1) ? dh : sh, (j & 1) ? dl : sl, A[i][j], B[i][j]);
+        }
     }
-    float* U = static_cast<float*>(a.U) + e;
+    // a unit is 2^t; the mean adds the centre sample
+    const int t = X - 1023 - 58 + 2 - up;
 #pragma unroll
     for (int j = 0; j < N1; ++j)
 #pragma unroll
         for (int i = 0; i < N1; ++i) {
-            const Split2& v = c[i][j / 2];
-            U[(i + N1 * j) * a.E] = (j & 1) ? v.hi.y + v.lo.y : v.hi.x + v.lo.x;
+            long long R = 4 * A[i][j] + ((B[i][j] + (1ll << 28)) >> 29);
+            if (neg) R = -R;
+            float v;
+            if (i + j == 0) v = (float)fma(__ll2double_rn(R), __hiloint2double((1023 + t) << 20, 0), f0);
+            else v = __ll2float_rn(R) * __int_as_float((127 - 50) << 23) * __int_as_float((127 + 50 + t) << 23);
+            U[(i + N1 * j) * a.E] = v;
         }
 }
 
@@ -1041,31 +1084,34 @@ static void project_tables(ProjArgs& a, int p, int nq)
 {
     double x[8], w[8];
     gauss_rule_public(nq, x, w);
+    // w_q P_i(g_q), and minv_i times it to 2^-60 from the exact product of the two doubles
+    auto set = [&](int q, int i, double P) {
+        a.WB[q][i] = w[q] * P;
+        const double lo = std::fma(w[q], P, -a.WB[q][i]);
+        const long long z = std::llrint(std::ldexp(a.WB[q][i], 60)) + std::llrint(std::ldexp(lo, 60));
+        const long long M = ((2 * i + 1) * z + 1) >> 1;
+        a.mh[q][i] = (int)((M + (1ll << 30)) >> 31);
+        a.ml[q][i] = (int)(M - ((long long)a.mh[q][i] << 31));
+    };
     for (int q = 0; q < nq; ++q) {
         double pm = 1.0, pc = x[q];
-        a.WB[q][0] = w[q];
-        a.WB[q][1] = w[q] * pc;
+        set(q, 0, 1.0);
+        set(q, 1, pc);
         for (int k = 1; k < p; ++k) {
             const double pn = ((2 * k + 1) * x[q] * pc - k * pm) / (k + 1);
             pm = pc; pc = pn;
-            a.WB[q][k + 1] = w[q] * pn;
+            set(q, k + 1, pn);
         }
     }
     for (int i = 0; i <= p; ++i) a.minv[i] = (2 * i + 1) / 2.0;
-    for (int q = 0; q < nq; ++q)
-        for (int i = 0; i <= p; ++i) {
-            const double v = a.minv[i] * a.WB[q][i];
-            a.sh[q][i] = (float)v;
-            a.sl[q][i] = (float)(v - (double)a.sh[q][i]);
-        }
 }
 
 template <int DIM, int N1, int NQ>
 static void launch_project_q(const ProjArgs& a, unsigned blocks, cudaStream_t s)
 {
-    if constexpr (DIM == 2) {
+    if constexpr (DIM == 2 && NQ >= 2) {     // (one point does not annihilate P_2)
         if (!a.f64) {
-            project_split_kernel<N1, NQ><<<blocks, 128, 0, s>>>(a);
+            project_fixed_kernel<N1, NQ><<<(unsigned)((a.E + kProjFixedThreads - 1) / kProjFixedThreads), kProjFixedThreads, 0, s>>>(a);
             return;
         }
     }
