@@ -79,7 +79,8 @@ struct dgw_ctx {
     void* adj_b1 = nullptr;      // adjoint: lambda of stage 2
     void* adj_b2 = nullptr;      // adjoint: lambda of stage 1
     std::map<std::pair<const void*, int>, bool> no_tmap;
-    // dgw_rk_step_host pipeline: streams for input copies, output copies and each stage; one event per (input copy or stage, band); the join events
+    // dgw_rk_step_host pipeline: streams for input copies, output copies and each stage; one
+    // event per (input copy or stage, band); the join events
     cudaStream_t band_st[2 + 3] = {};
     cudaEvent_t band_ev[4][16] = {};
     cudaEvent_t band_join[2] = {};

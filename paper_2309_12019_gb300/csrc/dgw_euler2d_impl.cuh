@@ -472,8 +472,8 @@ __global__ void __launch_bounds__(EX * EY, euler2_blocks<P>()) euler2d_kernel(co
                 } else {
                     const Real* a0 = A.Un + e + (int64_t)(2 * pr * K + k) * E;
                     const Real* a1 = a0 + (int64_t)K * E;
-                    unk.x = A.cg_loads ? __ldcg(a0) : *a0;
-                    unk.y = A.cg_loads ? __ldcg(a1) : *a1;
+                    unk.x = *a0;
+                    unk.y = *a1;
                 }
                 out = vfma(A.cn, unk, out);
             }

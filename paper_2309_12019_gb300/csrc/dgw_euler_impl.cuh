@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(TX, kF32 ? 8 : 4) euler_kernel(const __grid_co
 #pragma unroll
                 for (int k = 0; k < N1; ++k) {
                     const Real* a = usrc + (int64_t)(comp * N1 + k) * E;
-                    un[comp][k] = A.cg_loads ? __ldcg(a) : *a;
+                    un[comp][k] = *a;
                 }
         }
         put(c, tid + 1);

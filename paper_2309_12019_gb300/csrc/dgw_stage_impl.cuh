@@ -122,7 +122,6 @@ struct KParams {
     int use_tma;
     int use_tma_un;
     int use_p_un;        // the persistent kernel stages Un (tmap_un_p valid)
-    int cg_loads;        // load Uk / Un through L2 only (data written earlier in the same launch)
     int wait_limit;      // polls of a TMA mbarrier wait before it gives up (kWaitLimit)
     int tile_row0;       // first tile row of a stage launch over a band of rows
     int round_tiles;     // 2D Euler kernel: tiles that run at once (0: no prefetch of the next ones)
@@ -1119,22 +1118,22 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             row(qy, rr);
         }
     }
-            if (DIM == 2 && FLUX == FLUX_ROTATION && find_lam) {
-                // |v|^2 is convex, so over the Gauss points of the cell and of its faces it is largest at
-                // an outermost node of a face: the larger |v_x| and |v_y| of those four lines
-                const Real g = T.g[NQ - 1];
-                const Real vyg = max_pos(fabs(mul_x(A.omega, fma_x(A.hh, g, xc) - A.cx)), fabs(mul_x(A.omega, fma_x(A.hh, -g, xc) - A.cx)));
-                const Real vye = max_pos(fabs(mul_x(A.omega, fma_x(Real(gx), A.h, A.x0) - A.cx)),
-                                         fabs(mul_x(A.omega, fma_x(Real(gx + 1), A.h, A.x0) - A.cx)));
+    if (DIM == 2 && FLUX == FLUX_ROTATION && find_lam) {
+        // |v|^2 is convex, so over the Gauss points of the cell and of its faces it is largest at
+        // an outermost node of a face: the larger |v_x| and |v_y| of those four lines
+        const Real g = T.g[NQ - 1];
+        const Real vyg = max_pos(fabs(mul_x(A.omega, fma_x(A.hh, g, xc) - A.cx)), fabs(mul_x(A.omega, fma_x(A.hh, -g, xc) - A.cx)));
+        const Real vye = max_pos(fabs(mul_x(A.omega, fma_x(Real(gx), A.h, A.x0) - A.cx)),
+                                 fabs(mul_x(A.omega, fma_x(Real(gx + 1), A.h, A.x0) - A.cx)));
 #pragma unroll
-                for (int l = 0; l < L; ++l) {
-                    const Real yl = lane(yc, l);
-                    const Real vxg = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(A.hh, g, yl))), fabs(mul_x(A.omega, A.cy - fma_x(A.hh, -g, yl))));
-                    const Real vxe = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l]), A.h, A.y0))),
-                                             fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l] + 1), A.h, A.y0))));
-                    lane(lam, l) = max_pos(fma_x(vxg, vxg, mul_x(vye, vye)), fma_x(vxe, vxe, mul_x(vyg, vyg)));
-                }
-            }
+        for (int l = 0; l < L; ++l) {
+            const Real yl = lane(yc, l);
+            const Real vxg = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(A.hh, g, yl))), fabs(mul_x(A.omega, A.cy - fma_x(A.hh, -g, yl))));
+            const Real vxe = max_pos(fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l]), A.h, A.y0))),
+                                     fabs(mul_x(A.omega, A.cy - fma_x(Real(gy[l] + 1), A.h, A.y0))));
+            lane(lam, l) = max_pos(fma_x(vxg, vxg, mul_x(vye, vye)), fma_x(vxe, vxe, mul_x(vyg, vyg)));
+        }
+    }
     __syncthreads();
 
     // The stage array is no longer read: bring the Un tile into it now, so that its
@@ -1473,7 +1472,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
             for (int l = 0; l < L; ++l) {
                 const Real* un = A.Un + e[l] + k * E;
                 lane(unk, l) = (un_tma || un_async || un_pipe) ? sun[(k * TYC + cy[l]) * TX + lx]
-                                      : (in[l] ? (A.cg_loads ? __ldcg(un) : *un) : Real(0));
+                                      : (in[l] ? *un : Real(0));
             }
             out = vfma(A.cn, unk, out);
         }
@@ -1488,7 +1487,7 @@ __device__ __forceinline__ void process_tile(const KParams& A, const int tx0, co
 }
 
 // Resident CTAs per SM that the registers are sized for.  Float 2D: two (128 registers, no spills)
-// or, with `dense`, three at p = 2 (80, up to 24 bytes of spills) and four at p = 1 (64), for launches
+// or, with `dense`, three at p = 2 (80, 24 to 96 bytes of spills) and four at p = 1 (64), for launches
 // of more CTAs than that would leave in one round.  p = 2 FP32, us a stage, two / three CTAs: KPP 256^2
 // 10.2 / 12.4, 512^2 19.3 / 17.5, 1024^2 59.2 / 50.4; Burgers 512^2 25.5 / 25.9, 1024^2 68.2 / 60.2.
 // p = 1, three / four CTAs: Burgers 333 x 217 9.4 / 11.0, 1024^2 34.0 / 31.3.
@@ -1683,7 +1682,6 @@ static KParams make_params(const StageArgs& s)
     memset(&a, 0, sizeof a);
     a.use_tma = 0;
     a.use_tma_un = 0;
-    a.cg_loads = 0;
     a.wait_limit = s.wait_limit > 0 ? s.wait_limit : (s.wait_limit == 0 ? kWaitLimit : 0);
     a.tile_row0 = DIM == 2 ? s.tile_row0 : 0;
     if (s.tmap) {
@@ -1756,7 +1754,6 @@ __device__ __forceinline__ void batch_tiles(const BatchArgs& B, const BatchInst&
     KParams A;
     A.use_tma = 0;
     A.use_tma_un = 0;
-    A.cg_loads = 1;
     A.wait_limit = kWaitLimit;
     A.tile_row0 = 0;
     const Real* U = static_cast<const Real*>(B.U) + I.off;
