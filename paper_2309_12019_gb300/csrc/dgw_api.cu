@@ -917,8 +917,10 @@ __global__ void __launch_bounds__(128) project_kernel(const __grid_constant__ Pr
 // outside [2^-60, 2^100), take the sums in double.
 // The samples arrive through shared memory, whole lines at a time; 65 words a cell keep the lanes
 // that read one cell each on banks of their own.  1024^2 cells, p = 3, 8 x 8 samples, with the mass that
-// follows: every sample read K times in double 4.53 ms, project_cell in double 0.73 ms, this 0.29 ms
-// (604 MB would take 0.09 ms; the pipe of the 64-bit multiply-adds, 576 a cell, is 73 % busy).
+// follows: every sample read K times in double 4.53 ms, project_cell in double 0.73 ms, this 0.23 ms
+// (604 MB would take 0.09 ms).  The kernel alone takes 160 us: 2860 instructions a cell, 576 of them
+// 64-bit multiply-adds, issued in half of the slots by 12 warps per SM, which the samples in shared
+// memory hold it to.  Multiply-adds written in C took twice the instructions of their pipe (230 us).
 constexpr int kProjFixedThreads = 64;
 __device__ __forceinline__ void proj_limbs(long long x, int& h, int& l)
 {
@@ -928,9 +930,9 @@ __device__ __forceinline__ void proj_limbs(long long x, int& h, int& l)
 // A 2^62 + B 2^31 += (M x) 2^60
 __device__ __forceinline__ void proj_mad(int mh, int ml, int h, int l, long long& A, long long& B)
 {
-    A += (long long)mh * h;
-    B += (long long)mh * l;
-    B += (long long)ml * h;
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(A) : "r"(mh), "r"(h));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(B) : "r"(mh), "r"(l));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(B) : "r"(ml), "r"(h));
 }
 // v as an integer multiple (rounded down in magnitude) of 2^(X - 1023 - 58), X the largest biased
 // exponent of the cell
@@ -964,51 +966,57 @@ __global__ void __launch_bounds__(kProjFixedThreads) project_fixed_kernel(const 
 
     const double f0 = f[NQ / 2 * NQ + NQ / 2];
     const int h0 = __double2hiint(f0);
-    int top = 0, diff = 0;               // largest |f|; bits in which the upper words differ
+    // range of the upper words; one sign and exponent: they and all between share them
+    unsigned least = h0, most = h0;
 #pragma unroll
     for (int i = 0; i < NPT; ++i) {
-        const int h = __double2hiint(f[i]);
-        top = max(top, h & 0x7fffffff);
-        diff |= h ^ h0;
+        const unsigned h = (unsigned)__double2hiint(f[i]);
+        least = min(least, h);
+        most = max(most, h);
+    }
+    const bool same = ((least ^ most) >> 20) == 0;
+    int top = (int)(most & 0x7fffffffu);     // largest |f|
+    if (!same) {
+        for (int i = 0; i < NPT; ++i) top = max(top, __double2hiint(f[i]) & 0x7fffffff);
     }
     const int X = top >> 20;
     if (X != 0 && (X < 1023 - 60 || X >= 1023 + 100)) {
         project_cell<2, N1, NQ>(a, e);
         return;
     }
-    int bits = 0;                        // set bits of the upper words of |d|
-    int neg = 0;                         // d is taken of -f
-    if ((diff & 0xfff00000) == 0) {
-        // one sign and exponent (or all zero): the difference of the bits is that of the significands
-        const long long b0 = __double_as_longlong(f0);
+    // d = x - base, x the words in shared memory, in units of 2^unit; of -f where neg
+    long long base = 0;
+    int unit = X - 1023 - 58, len;           // |d| <= 2^len
+    bool neg = false, exact = true;
+    if (same) {
+        // the differences of the bits are those of the significands
+        base = __double_as_longlong(f0);
+        unit = X - 1023 - 52;
         neg = h0 < 0;
-#pragma unroll 16
-        for (int i = 0; i < NPT; ++i) {
-            const long long q = (d[i] - b0) * 64;
-            const int h = (int)(q >> 32);
-            bits |= h ^ (h >> 31);
-            d[i] = q;
-        }
+        const unsigned far = max(most - (unsigned)h0, (unsigned)h0 - least);
+        exact = far == 0;                    // (the upper words do not tell)
+        len = 64 - __clz(far);
     } else {
         const long long q0 = proj_fixed(f0, X);
 #pragma unroll 8
-        for (int i = 0; i < NPT; ++i) {
-            const long long q = proj_fixed(f[i], X) - q0;
-            const int h = (int)(q >> 32);
-            bits |= h ^ (h >> 31);
-            d[i] = q;
-        }
+        for (int i = 0; i < NPT; ++i) d[i] = proj_fixed(f[i], X) - q0;
     }
-    unsigned long long mask = (unsigned long long)(unsigned)bits << 32;
-    if (bits == 0)                       // (all below 2^-27 of the largest sample)
-        for (int i = 0; i < NPT; ++i) mask |= (unsigned long long)(d[i] ^ (d[i] >> 63));
-    if (mask == 0 || X == 0) {           // a constant, or nothing but zeros and numbers below the normal ones
+    if (exact) {
+        long long mask = 0;
+        for (int i = 0; i < NPT; ++i) {
+            const long long q = d[i] - base;
+            mask |= q ^ (q >> 63);
+        }
+        len = 64 - __clzll(mask);
+    }
+    if (len == 0 || X == 0) {                // a constant, or nothing but zeros and numbers below the normal ones
 #pragma unroll
         for (int k = 0; k < N1 * N1; ++k) U[k * a.E] = k == 0 ? (float)f0 : 0.f;
         return;
     }
-    const int up = __clzll((long long)mask) - 4;
-    auto shl = [up](long long v) { return (long long)((unsigned long long)v << up); };
+    const int up = 60 - len;
+    using u64 = unsigned long long;
+    auto get = [d](int i) { return (u64)d[i]; };
 
     long long A[N1][N1], B[N1][N1];
 #pragma unroll
@@ -1022,17 +1030,17 @@ __global__ void __launch_bounds__(kProjFixedThreads) project_fixed_kernel(const 
         for (int i = 0; i < N1; ++i) ra[i] = rb[i] = 0;
         if constexpr ((NQ & 1) != 0) {
             int h, l;
-            proj_limbs(shl(d[b * NQ + NP]), h, l);
+            proj_limbs((long long)((get(b * NQ + NP) - (u64)base) << up), h, l);
 #pragma unroll
             for (int i = 0; i < N1; i += 2) proj_mad(a.mh[NP][i], a.ml[NP][i], h, l, ra[i], rb[i]);
         }
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             const int qp = NQ - 1 - q;
-            const long long x = shl(d[b * NQ + qp]), y = shl(d[b * NQ + q]);
+            const u64 x = get(b * NQ + qp), y = get(b * NQ + q);
             int sh, sl, dh, dl;
-            proj_limbs(x + y, sh, sl);
-            proj_limbs(x - y, dh, dl);
+            proj_limbs((long long)((x + y - 2 * (u64)base) << up), sh, sl);
+            proj_limbs((long long)((x - y) << up), dh, dl);
 #pragma unroll
             for (int i = 0; i < N1; ++i) proj_mad(a.mh[qp][i], a.ml[qp][i], (i & 1) ? dh : sh, (i & 1) ? dl : sl, ra[i], rb[i]);
         }
@@ -1066,7 +1074,7 @@ __global__ void __launch_bounds__(kProjFixedThreads) project_fixed_kernel(const 
         }
     }
     // a unit is 2^t; the mean adds the centre sample
-    const int t = X - 1023 - 58 + 2 - up;
+    const int t = unit + 2 - up;
 #pragma unroll
     for (int j = 0; j < N1; ++j)
 #pragma unroll
