@@ -176,7 +176,8 @@ dgw_status dgw_set_params(dgw_ctx* ctx, const dgw_params* params);
 /* L2 projection of initial data onto V_p (Sec. 2, Eq. fesol).  samples (device,
  * double, E * nq^dim values): f at the nq-point Gauss-Legendre points of each
  * element, sample t = a + nq*b at x = xc + h/2 g_a, y = yc + h/2 g_b.  nq in 1..8.
- * U (device, context precision, K*E) receives c_k = int f phi_k / int phi_k^2.  Euler
+ * U (device, context precision, K*E) receives c_k = int f phi_k / int phi_k^2: sums in
+ * double or of at least its accuracy, rounded once to the context's precision.  Euler
  * system: (dim + 2) * E * nq^dim samples, those of each conserved variable one after
  * the other. */
 dgw_status dgw_project(dgw_ctx* ctx, int nq, const double* samples, void* U, void* stream);
